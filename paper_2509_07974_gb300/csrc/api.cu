@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "basis.cuh"
 #include "common.cuh"
 
 namespace ext4pcf {
@@ -125,6 +126,7 @@ struct ext4pcf_ctx {
   // tensor-core contraction: work items (built once per shape) and the device status word
   DBuf tc_items, tc_xb, tc_red, tc_rowmax, status, geom;
   int tc_N = -1, tc_nb = -1;
+  ext4pcf::Basis basis{};  // rows of the reduced array for the last (n_max, n_bins)
   size_t tc_items_bytes = 0;
   cudaEvent_t ev[8] = {};
   std::vector<cudaEvent_t> tev;  // per-phase timing events of one measure call (grown on demand)
@@ -444,6 +446,11 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
       ctx->tc_N = n_max;
       ctx->tc_nb = n_bins;
     }
+  }
+  // the FP64 and FP32 forms collect the independent sums of one output slot at a time
+  const bool cc = !tc && !records;
+  if (cc && (ctx->basis.N != n_max || ctx->basis.nb != n_bins || ctx->basis.npairs == 0)) {
+    if (!basis_make(L, ctx->basis)) return fail(ctx, EXT4PCF_E_UNSUPPORTED, "no reduced rows for this n_max");
   }
   const long long timeout = ctx->cfg.timeout_cycles > 0 ? ctx->cfg.timeout_cycles : 20000000000LL;
 
@@ -803,6 +810,12 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
     ENSURE(ctx->tc_red, red_doubles * 8 * n_out);
     CK(cudaMemsetAsync(ctx->tc_red.p, 0, red_doubles * 8 * n_out, s));
   }
+  const int cc_slices = cc ? contract_slices(ctx->basis) : 1;
+  const size_t cc_bytes = cc ? ctx->basis.elems() * 16 * cc_slices : 0;
+  if (cc) {
+    ENSURE(ctx->tc_red, cc_bytes);
+    CK(cudaMemsetAsync(ctx->tc_red.p, 0, cc_bytes, s));
+  }
   // Wave planner: the catalogues' centre lists in order.  With `multi`, a wave packs runs of
   // several lists whose lengths are known on the host, each starting at a multiple of 64
   // records; otherwise (or for a list counted on the device) a wave is one run of one list.
@@ -848,6 +861,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   size_t wave_i = 0;
   WavePlan P;
   double* red_base = (double*)ctx->tc_red.p;
+  int red_slot = -1;  // output slot of the CUDA-core forms' reduced array
   double* corr_base = (double*)ctx->corr.p;
   for (;;) {
     const bool tuning = wave_i < trial.size();
@@ -883,12 +897,19 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
       continue;
     }
     if (timing) t_w1 = tmark();
+    if (cc && g0.slot != red_slot) {  // the next slot: the last one's sums go to its output
+      if (red_slot >= 0) {
+        CK(basis_expand(ctx->basis, red_base, cc_slices, d_ups + 2 * ups_elems * (size_t)red_slot, s));
+        CK(cudaMemsetAsync(red_base, 0, cc_bytes, s));
+      }
+      red_slot = g0.slot;
+    }
     if (f64) {
-      CK(contract_wave<double>(L, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, g0.t, g0.n_live, g0.w0,
-                               d_ups + 2 * ups_elems * (size_t)g0.slot, s));
+      CK(contract_wave<double>(L, ctx->basis, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, g0.t, g0.n_live,
+                               g0.w0, red_base, s));
     } else if (prec == EXT4PCF_FP32) {
-      CK(contract_wave<float>(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, g0.t, g0.n_live, g0.w0,
-                              d_ups + 2 * ups_elems * (size_t)g0.slot, s));
+      CK(contract_wave<float>(L, ctx->basis, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, g0.t, g0.n_live,
+                              g0.w0, red_base, s));
     } else if (prec == EXT4PCF_SPLIT_F16) {
       CK(contract_wave_h16(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, red_base,
                            (const int4*)ctx->tc_items.p, (int)(ctx->tc_items_bytes / sizeof(int4)),
@@ -931,6 +952,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   ctx->last_wave = std::min(T, largest_wave);  // the wave size in use (trial waves aside)
   if (records && rec_host && n_rec > 0)
     CK(cudaMemcpyAsync(rec_out, ctx->rec_out.p, (size_t)n_rec * L.rec * 16, cudaMemcpyDeviceToHost, s));
+  if (red_slot >= 0) CK(basis_expand(ctx->basis, red_base, cc_slices, d_ups + 2 * ups_elems * (size_t)red_slot, s));
   // ---- per output slot: every ordered triple from the reduced array, then the corrections
   for (int o = 0; o < n_out && !records; ++o) {
     double* ups_o = d_ups + 2 * ups_elems * (size_t)o;

@@ -236,10 +236,11 @@ cudaError_t gather_wave(const SortedCat& cat, const SortedCat& cen, const Bins& 
                         const WavePlan& plan, bool accumulate, cplx_t<R>* rec, cplx_t<R>* xw,
                         unsigned long long* pair_count, int sm_count, cudaStream_t s);
 
-// contract.cu
+// contract.cu: a wave's independent sums (basis.cuh), added into the reduced array of its slot
+struct Basis;
 template <typename R>
-cudaError_t contract_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t<R>* xw, int T,
-                          const int* n_live, int w0, double* ups, cudaStream_t s);
+cudaError_t contract_wave(const Layout& L, const Basis& B, const cplx_t<R>* rec, const cplx_t<R>* xw, int T,
+                          const int* n_live, int w0, double* red, cudaStream_t s);
 // correction sums of every segment into its slot: corr + slot * corrections_size(L), and
 // (xi_acc non-null) xi_acc + slot * 6 nb
 template <typename R>
