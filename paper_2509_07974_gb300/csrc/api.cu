@@ -436,21 +436,24 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   // waves that pack the centres of several catalogues: the split-FP16 contraction, the gather
   // and the correction sums take segments; the other contraction forms one catalogue a wave
   const bool multi = prec == EXT4PCF_SPLIT_F16;
+  // the FP64 and FP32 forms collect the independent sums (basis.cuh) of one output slot at a
+  // time, the split-FP16 form those of every slot
+  const bool cc = !tc && !records;
+  const bool h16 = prec == EXT4PCF_SPLIT_F16;
+  if ((cc || h16) && (ctx->basis.N != n_max || ctx->basis.nb != n_bins || ctx->basis.npairs == 0)) {
+    if (!basis_make(L, ctx->basis)) return fail(ctx, EXT4PCF_E_UNSUPPORTED, "no reduced rows for this n_max");
+  }
   if (tc) {
     if (ctx->tc_N != n_max || ctx->tc_nb != n_bins) {
       std::vector<int4> items;
-      if (!tc_build_items(L, items)) return fail(ctx, EXT4PCF_E_UNSUPPORTED, "no symmetry map for the contraction table");
+      if (h16) h16_build_items(ctx->basis, items);
+      else if (!tc_build_items(L, items)) return fail(ctx, EXT4PCF_E_UNSUPPORTED, "no symmetry map for the contraction table");
       ENSURE(ctx->tc_items, items.size() * sizeof(int4));
       CK(cudaMemcpy(ctx->tc_items.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
       ctx->tc_items_bytes = items.size() * sizeof(int4);
       ctx->tc_N = n_max;
       ctx->tc_nb = n_bins;
     }
-  }
-  // the FP64 and FP32 forms collect the independent sums of one output slot at a time
-  const bool cc = !tc && !records;
-  if (cc && (ctx->basis.N != n_max || ctx->basis.nb != n_bins || ctx->basis.npairs == 0)) {
-    if (!basis_make(L, ctx->basis)) return fail(ctx, EXT4PCF_E_UNSUPPORTED, "no reduced rows for this n_max");
   }
   const long long timeout = ctx->cfg.timeout_cycles > 0 ? ctx->cfg.timeout_cycles : 20000000000LL;
 
@@ -805,7 +808,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   const size_t corr_doubles = corrections_size(L);
   ENSURE(ctx->corr, corr_doubles * 8 * n_out);
   CK(cudaMemsetAsync(ctx->corr.p, 0, corr_doubles * 8 * n_out, s));
-  const size_t red_doubles = tc ? tc_reduced_doubles(L) : 0;
+  const size_t red_doubles = h16 ? 2 * ctx->basis.elems() : tc ? tc_reduced_doubles(L) : 0;
   if (tc) {
     ENSURE(ctx->tc_red, red_doubles * 8 * n_out);
     CK(cudaMemsetAsync(ctx->tc_red.p, 0, red_doubles * 8 * n_out, s));
@@ -910,8 +913,8 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
     } else if (prec == EXT4PCF_FP32) {
       CK(contract_wave<float>(L, ctx->basis, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, g0.t, g0.n_live,
                               g0.w0, red_base, s));
-    } else if (prec == EXT4PCF_SPLIT_F16) {
-      CK(contract_wave_h16(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, red_base,
+    } else if (h16) {
+      CK(contract_wave_h16(L, ctx->basis, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, red_base,
                            (const int4*)ctx->tc_items.p, (int)(ctx->tc_items_bytes / sizeof(int4)),
                            (float2*)ctx->tc_xb.p, (unsigned*)ctx->tc_rowmax.p, (int*)ctx->status.p, timeout, s));
     } else {
@@ -956,7 +959,8 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   // ---- per output slot: every ordered triple from the reduced array, then the corrections
   for (int o = 0; o < n_out && !records; ++o) {
     double* ups_o = d_ups + 2 * ups_elems * (size_t)o;
-    if (tc) CK(tc_expand(L, red_base + red_doubles * (size_t)o, ups_o, s));
+    if (h16) CK(basis_expand(ctx->basis, red_base + red_doubles * (size_t)o, 1, ups_o, s));
+    else if (tc) CK(tc_expand(L, red_base + red_doubles * (size_t)o, ups_o, s));
     CK(corrections_apply(L, corr_base + corr_doubles * (size_t)o, ups_o, s));
   }
   if (host_ups) CK(cudaMemcpyAsync(upsilon, d_ups, ups_bytes * n_out, cudaMemcpyDeviceToHost, s));

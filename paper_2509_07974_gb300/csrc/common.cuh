@@ -267,9 +267,11 @@ cudaError_t tc_expand(const Layout& L, const double* red, double* ups, cudaStrea
 bool h16_supported(const Layout& L);
 size_t contract_h16_wave_bytes(const Layout& L, int T);
 size_t contract_h16_rowmax_bytes(const Layout& L);
-// (plan: every segment's sums go to red + slot * tc_reduced_doubles(L))
-cudaError_t contract_wave_h16(const Layout& L, const float2* rec, const float2* xw, const WavePlan& plan,
-                              double* red, const int4* items, int n_items, float2* wave, unsigned* rowmax,
-                              int* status, long long timeout, cudaStream_t s);
+void h16_build_items(const Basis& B, std::vector<int4>& items);
+// (plan: every segment's sums go to its slot's reduced array of the independent sums, red +
+// slot * 2 * B.elems() doubles)
+cudaError_t contract_wave_h16(const Layout& L, const Basis& B, const float2* rec, const float2* xw,
+                              const WavePlan& plan, double* red, const int4* items, int n_items, float2* wave,
+                              unsigned* rowmax, int* status, long long timeout, cudaStream_t s);
 
 }  // namespace ext4pcf

@@ -1,46 +1,48 @@
 // Split-FP16 tensor-core contraction of a wave (tcgen05 kind::f16, sm_103a).
 //
-// The GEMM is that of the other tensor-core forms (contract_tc.cu): for fixed s = n2 + n3 the
-// Khatri-Rao rows x~B[n2](Th2) C[n3](Th3) over the bin pairs Th2 <= Th3 are multiplied with the
-// column factors A^mu[s](Th1), K running over the centres, and the sums go to the reduced array
-// of the Theta2 <-> Theta3 symmetry (Table tab:4PCFSymm).  This kernel arranges the data so
-// that forming the rows on the CUDA cores -- the part that bounds the other forms -- takes
-// about as long as the tensor core's three passes:
+// The GEMM runs over the independent sums of basis.cuh: for fixed sg the row products
+// G_a(b2) G_{sg-a}(b3), b2 <= b3, are multiplied with the columns x G_{-sg-8}(b1), x^* G_{-sg-4}(b1),
+// x G_{sg+4}^*(b1) and x^* G_sg^*(b1) (families F0..F3; W rows with the column w W_{-sg}), K running
+// over the centres.  Every row product serves four families, so 1643 tiles of 128 rows (n_max = 20,
+// 10 bins) hold what took 5572 tiles with a row type per component.  Forming the rows on the CUDA
+// cores is the larger part of the work.  One wave of 8192 centres at these sizes: 6.5 -> 2.24 ms
+// (3300 clocks per 64-centre stage of a tile, of which shared memory is busy for about 2750: row
+// products read 1024 wavefronts, the columns' embedding moves 480, the MMAs read 480 and the bulk
+// copies write 480).  The data are arranged for the producers:
 //  * Power-of-two row scales.  A pre-pass finds the largest |component| of every row of the
-//    wave array (x~B, G, W rows) and the transpose writes each row times 2^k, its largest
-//    component in [2^6, 2^7).  A product of two rows is then below 2^15, inside the fp16
-//    range, with no per-value scaling in the kernel; the epilogue takes out the exact factor
-//    2^-(k_B + k_C + k_A).
-//  * Planar staging.  Per 16 centres a row holds their 16 real parts, then their 16 imaginary
-//    parts (128 bytes), so that two centres' real (or imaginary) parts form one 64-bit register
-//    pair and the complex products run on the packed f32x2 pipe.
-//  * Stage-major wave array.  The array is laid out [stage of 64 centres][row][512 bytes], the
-//    16-byte chunks of every 128-byte quarter XOR-permuted by the row index mod 8 (the 128-byte
-//    swizzle, applied by the transpose).  The rows a work item needs for one stage (its x~B,
-//    C and A blocks) are then four contiguous ranges, fetched with four plain bulk copies
+//    wave array and the transpose writes each row times 2^k, its largest component in
+//    [2^6, 2^7).  A product of two rows is then below 2^15, inside the fp16 range, with no
+//    per-value scaling in the kernel; the epilogue takes out the exact factor in FP64.
+//  * Planar staging.  Per 16 centres a G or W row holds their 16 real parts, then their 16
+//    imaginary parts (128 bytes), so that two centres' real (or imaginary) parts form one 64-bit
+//    register pair and the complex products run on the packed f32x2 pipe.  The column rows
+//    (x G, x^* G, w W) are split into fp16 hi and lo by the transpose: real hi | imaginary hi |
+//    real lo | imaginary lo, 64 centres each.
+//  * Stage-major wave array.  The array is laid out [stage of 64 centres][row][512 bytes]; in
+//    the G and W rows the 16-byte chunks of every 128-byte quarter are XOR-permuted by the row
+//    index mod 8 (the 128-byte swizzle, applied by the transpose).  The rows a work item needs
+//    for one stage are six contiguous ranges, fetched with six plain bulk copies
 //    (cp.async.bulk) instead of one tensor box per 8 rows and 16 centres: the copy engine's
 //    per-request cost, not bandwidth, bounded the boxed staging.  Eight lanes reading eight
 //    consecutive rows at the same logical chunk hit eight different bank groups.
 //  * K order.  In every group of 8 centres (one MMA, K = 16 halves) K = 0..7 holds the real
-//    and K = 8..15 the imaginary parts of the row values; the column operand holds (A_r, -A_i)
-//    for the real and (A_i, A_r) for the imaginary output at the same K.
-//  * W for both signs of m.  W_{-m} = conj W_m is written out, so the conjugation of every
-//    factor is fixed by the row type and uniform over a work item.
+//    and K = 8..15 the imaginary parts.
 //  * 64-centre stages and ring counters without divisions: each producer thread forms 16
-//    values of its row per stage between two barrier crossings.
+//    values of its row per stage between two barrier crossings; two warps of their own write
+//    the columns' real embedding (the B operand).
 // Precision: every operand is split into fp16 hi + lo (22 significant bits) and the MMAs
-// accumulate hi*hi + hi*lo + lo*hi in FP32 over one stage; the stage's partial sums are
+// accumulate hi*lo + lo*hi + hi*hi in FP32 over one stage; the stage's partial sums are
 // promoted into FP32 registers while the next stage runs, and the epilogue adds them into the
 // FP64 reduced array.
 // Every wait is bounded by a clock budget; on expiry the kernel records an error code, runs to
 // its end, waits for its own MMAs and copies and frees its TMEM.
 #include <cuda.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <vector>
 
-#include "common.cuh"
-#include "kr_table.cuh"
+#include "basis.cuh"
 #include "tc_ptx.cuh"
 
 namespace ext4pcf {
@@ -49,11 +51,12 @@ namespace {
 
 constexpr int kHCentres = 64;                        // centres per stage
 constexpr int kHProducerWarps = 16;
-constexpr int kHThreads = kHProducerWarps * 32 + 64; // + the MMA issuer and the TMA loader warp
-constexpr int kHWarpMma = kHProducerWarps, kHWarpLoad = kHProducerWarps + 1;
-constexpr int kHSlots = 3;                           // A (TMEM) and B (shared) ring depth
+constexpr int kHColumnWarps = 2;
+constexpr int kHWarpMma = kHProducerWarps + kHColumnWarps, kHWarpLoad = kHWarpMma + 1;
+constexpr int kHThreads = (kHWarpLoad + 1) * 32;
+constexpr int kHArrivals = kHProducerWarps + kHColumnWarps;
 constexpr int kHACols = 128;                         // TMEM columns per A slot: 64 hi + 64 lo
-constexpr int kHDCols = 128;                         // two D buffers of 64 columns
+constexpr int kHMaxSlots = 3;                        // A (TMEM) and B (shared) ring depth at most
 constexpr int kHMaxIn = 4;                           // staged-input ring depth at most
 constexpr uint32_t kHTmemCols = 512;
 constexpr int kHScaleTop = 6;                        // rows scaled into [2^6, 2^7)
@@ -73,32 +76,41 @@ __host__ __device__ __forceinline__ int h_scale_exp(unsigned mbits) {
 __device__ __forceinline__ float h_pow2f(int k) { return __int_as_float((127 + k) << 23); }
 __device__ __forceinline__ double h_pow2d(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
 
-// Row of the transposed wave array at one centre (rc: the centre's record, x = w gamma, w):
-//   rows [0, row_g)      x~B per x~B type: (type, n2 + N + 1, bin), n2 in [-N-1, N+1]
-//   rows [row_g, row_w)  G_n(bin), n in [-2N-3, 2N-1]
-//   rows [row_w, rows)   W_m(bin), m in [-2N, 2N]
-__device__ __forceinline__ float2 hwave_value(const Layout& L, const float2* __restrict__ rc, float2 x, float w,
-                                              int r, int row_g, int row_w) {
-  const int nb = L.nb, N = L.N, nx = 2 * N + 3;
-  if (r >= row_w) {
-    const int m = (r - row_w) / nb - 2 * N, b = (r - row_w) % nb;
+// Rows of the transposed wave array:
+//   [0, w)       G_m(bin), m in [-2N-3, 2N-1]
+//   [w, xg)      W_m(bin), m in [-2N, 2N]
+//   [xg, xcg)    x G_m(bin)       (column rows, split into fp16 hi and lo)
+//   [xcg, ww)    x^* G_m(bin)
+//   [ww, rows)   w W_m(bin), m in [0, 2N]
+struct HRows {
+  int w, xg, xcg, ww, rows;
+  __host__ __device__ static HRows make(const Layout& L) {
+    HRows r;
+    r.w = L.nG * L.nb;
+    r.xg = r.w + (4 * L.N + 1) * L.nb;
+    r.xcg = r.xg + L.nG * L.nb;
+    r.ww = r.xcg + L.nG * L.nb;
+    r.rows = r.ww + L.nW * L.nb;
+    return r;
+  }
+};
+// value of row r at one centre (rc: the centre's record, x = w gamma, w)
+__device__ __forceinline__ float2 hwave_value(const Layout& L, const HRows& R, const float2* __restrict__ rc, float2 x,
+                                              float w, int r) {
+  const int nb = L.nb;
+  if (r < R.w) return rc[L.oG + r];
+  if (r < R.xg) {
+    const int m = (r - R.w) / nb - 2 * L.N, b = (r - R.w) % nb;
     float2 f = rc[L.W(m >= 0 ? m : -m, b)];
     if (m < 0) f.y = -f.y;
     return f;
   }
-  if (r >= row_g) return rc[L.oG + (r - row_g)];
-  const int t = r / (nx * nb), n2 = (r / nb) % nx - N - 1, b = r % nb;
-  float2 f;
-  if (t == 4) {
-    const int m = -n2;  // w W[-n2], |n2| <= N
-    f = (m <= N && m >= -N) ? rc[L.W(m >= 0 ? m : -m, b)] : make_float2(0.f, 0.f);
-    if (m < 0) f.y = -f.y;
-    x = make_float2(w, 0.f);
-  } else {
-    f = (t & 1) ? rc[L.G(n2 - 2, b)] : rc[L.G(-n2 - 2, b)];
-    if (t & 1) f.y = -f.y;
-    if (t >= 2) x.y = -x.y;
+  if (r >= R.ww) {
+    const float2 f = rc[L.oW + (r - R.ww)];
+    return make_float2(w * f.x, w * f.y);
   }
+  if (r >= R.xcg) x.y = -x.y;
+  const float2 f = rc[L.oG + (r >= R.xcg ? r - R.xcg : r - R.xg)];
   return make_float2(x.x * f.x - x.y * f.y, x.x * f.y + x.y * f.x);
 }
 
@@ -106,43 +118,41 @@ __device__ __forceinline__ float2 hwave_value(const Layout& L, const float2* __r
 // (records of the wave's live centres only: padding records are never read)
 __global__ void __launch_bounds__(256) hwave_rowmax_kernel(const Layout L, const float2* __restrict__ rec,
                                                            const float2* __restrict__ xw, const WavePlan plan,
-                                                           int row_g, int row_w, int rows,
-                                                           unsigned* __restrict__ rowmax) {
+                                                           const HRows R, unsigned* __restrict__ rowmax) {
   __shared__ float part[8][33];
   const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 128;
   if (c0 >= plan.total) return;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, r = r0 + tx;
   float m = 0.f;
-  if (r < rows) {
+  if (r < R.rows) {
     for (int k = 0; k < 16; ++k) {
       const int c = c0 + ty + 8 * k;
       int j = 0;
       const int si = c < plan.total ? seg_of(plan, c, &j) : -1;
       if (si >= 0 && j < seg_live(plan.seg[si])) {
-        const float2 v = hwave_value(L, rec + (size_t)c * L.rec, xw[2 * (size_t)c], xw[2 * (size_t)c + 1].x, r,
-                                     row_g, row_w);
+        const float2 v = hwave_value(L, R, rec + (size_t)c * L.rec, xw[2 * (size_t)c], xw[2 * (size_t)c + 1].x, r);
         m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
       }
     }
   }
   part[ty][tx] = m;
   __syncthreads();
-  if (ty == 0 && r < rows) {
+  if (ty == 0 && r < R.rows) {
     for (int k = 1; k < 8; ++k) m = fmaxf(m, part[k][tx]);
     if (m > 0.f) atomicMax(&rowmax[r], __float_as_uint(m));  // non-negative floats order as integers
   }
 }
 
-// The transposed, scaled, planar wave array, stage-major: record c of row r sits in stage
-// c / 64 at float (c / 64 * rows + r) * 128 + q * 32 + ((k ^ (r % 8)) * 4) + c % 4, with
-// q = (c % 64) / 16 the quarter and k = (c % 16) / 4 (real part) or 4 + (c % 16) / 4
-// (imaginary part) the logical 16-byte chunk.
+// The transposed, scaled wave array, stage-major: record c of row r sits in stage c / 64, in the
+// 512 bytes of row r there.  G and W rows: float q * 32 + ((k ^ (r % 8)) * 4) + c % 4 with
+// q = (c % 64) / 16 the quarter and k = (c % 16) / 4 (real part) or 4 + (c % 16) / 4 (imaginary
+// part) the logical 16-byte chunk.  Column rows: half c % 64 of each of the four planes real hi,
+// imaginary hi, real lo, imaginary lo.
 // Padding records (between segments, past a segment's live centres, past the wave up to a
 // multiple of 64) are written as zeros.
 __global__ void __launch_bounds__(256) hwave_transpose_kernel(const Layout L, const float2* __restrict__ rec,
                                                               const float2* __restrict__ xw, const WavePlan plan,
-                                                              int row_g, int row_w, int rows,
-                                                              const unsigned* __restrict__ rowmax,
+                                                              const HRows R, const unsigned* __restrict__ rowmax,
                                                               float* __restrict__ out) {
   __shared__ float2 tile[32][33];
   const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
@@ -155,90 +165,100 @@ __global__ void __launch_bounds__(256) hwave_transpose_kernel(const Layout L, co
     float2 v = make_float2(0.f, 0.f);
     int j = 0;
     const int si = c < plan.total ? seg_of(plan, c, &j) : -1;
-    if (si >= 0 && j < seg_live(plan.seg[si]) && r < rows)
-      v = hwave_value(L, rec + (size_t)c * L.rec, xw[2 * (size_t)c], xw[2 * (size_t)c + 1].x, r, row_g, row_w);
+    if (si >= 0 && j < seg_live(plan.seg[si]) && r < R.rows)
+      v = hwave_value(L, R, rec + (size_t)c * L.rec, xw[2 * (size_t)c], xw[2 * (size_t)c + 1].x, r);
     tile[ty + 8 * k][tx] = v;
   }
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int r = r0 + ty + 8 * k, c = c0 + tx;
-    if (r < rows) {
-      const float sc = h_pow2f(h_scale_exp(rowmax[r]));
-      const float2 v = tile[tx][ty + 8 * k];
+    if (r >= R.rows) continue;
+    const float sc = h_pow2f(h_scale_exp(rowmax[r]));
+    float2 v = tile[tx][ty + 8 * k];
+    v.x *= sc;
+    v.y *= sc;
+    float* row = out + ((size_t)(c >> 6) * R.rows + r) * 128;
+    if (r >= R.xg) {
+      __half* h = reinterpret_cast<__half*>(row) + (c & 63);
+      const __half xh = __float2half_rn(v.x), yh = __float2half_rn(v.y);
+      h[0] = xh;
+      h[64] = yh;
+      h[128] = __float2half_rn(v.x - __half2float(xh));
+      h[192] = __float2half_rn(v.y - __half2float(yh));
+    } else {
       const int q = (c & 63) >> 4, kre = (c & 15) >> 2, sw = r & 7;
-      float* o = out + ((size_t)(c >> 6) * rows + r) * 128 + q * 32 + (c & 3);
-      o[(kre ^ sw) * 4] = v.x * sc;
-      o[((4 + kre) ^ sw) * 4] = v.y * sc;
+      float* o = row + q * 32 + (c & 3);
+      o[(kre ^ sw) * 4] = v.x;
+      o[((4 + kre) ^ sw) * 4] = v.y;
     }
   }
 }
 
 struct HArgs {
   Layout L;
+  HRows R;
   WavePlan plan;      // the wave's segments (a segment starts at a stage boundary)
-  double* red;        // reduced outputs [slot][9][2N+3][2N+3][nb][npairs] (complex, FP64)
-  size_t red_stride;  // doubles per slot
+  double2* red;       // reduced outputs, one array (basis.cuh) per slot
+  size_t red_stride;  // complex elements per slot
+  size_t red_w;       // first W element
   int npairs;
-  const int4* items;  // (type, s, row0, nrows | (n2 of row 0 of the s block + 64) << 8)
+  const int4* items;  // kind | group << 1 | (first a of sg + 128) << 8 | rows << 16, sg, first row, row base
   int n_items;
-  int row_g, row_w;   // first G row and first W row of the wave array
+  int ncomp;          // families per X item: 4, or 2 in two groups (F0, F2 and F1, F3)
   const unsigned* rowmax;  // largest |component| per row (float bits): the row scales
   const float* wave;  // the stage-major wave array
-  int rows;           // its rows
   int in_stages;      // staged-input ring depth
   int stage_rows;     // rows per staged stage
-  int npad_max;       // rows of a B tile: 2 * 2 * nb rounded up to 16
+  int npad_max;       // rows of a B tile
   long long timeout;
   int* status;
 };
 
-// rows of factor f for its variable in [va, vb]: first row in the wave array, count, and the
-// multipole index of the first row
-struct HBlk {
-  int row0, len, lo;
-};
-__device__ __forceinline__ HBlk hblk(const HArgs& a, KF f, int va, int vb) {
-  const int nb = a.L.nb, N = a.L.N;
-  const int nlo = f.sgn > 0 ? va + f.off : -vb + f.off;
-  const int nhi = f.sgn > 0 ? vb + f.off : -va + f.off;
-  HBlk b;
-  b.lo = nlo;
-  b.len = (nhi - nlo + 1) * nb;
-  b.row0 = f.arr == 0 ? a.row_g + (nlo + 2 * N + 3) * nb : a.row_w + (nlo + 2 * N) * nb;
-  return b;
-}
-__device__ __forceinline__ int hblk_index(const HBlk& k, KF f, int v, int b, int nb) {
-  return (f.sgn * v + f.off - k.lo) * nb + b;
-}
-
-// Geometry of one work item: the staged blocks (x~B rows, C rows, A rows) and their first
-// rows in a staged stage (packed one after the other)
+// Geometry of one work item: the staged blocks (first rows of the wave array, rows) and where they
+// sit in a staged stage, packed one after the other: the G_a (W_a) rows, the G_{sg-a} rows, then nb
+// rows per column family
 struct HGeo {
-  int s, row0, nrows, n2a, t2a, t2b;
-  HBlk bx, bc, ba0, ba1;
-  int sx, sc, sa0, sa1;
+  bool w;
+  int sg, row0, nrows, alo, base;
+  int a1, a2, m1;   // the tile's a range, and the first index of the second block
+  int blk2, blk3;   // first rows of the wave array
+  int len;          // rows of each of the two blocks
+  int nfam;         // column families
 };
-__device__ __forceinline__ HGeo hgeo(const HArgs& a, int4 item, const KRType& kr) {
-  const int nb = a.L.nb, N = a.L.N, nx = 2 * N + 3;
+__device__ __forceinline__ HGeo hgeo(const HArgs& a, int4 item) {
+  const int nb = a.L.nb, N = a.L.N;
   HGeo g;
-  g.s = item.y;
+  g.w = (item.x & 1) != 0;
+  g.sg = item.y;
   g.row0 = item.z;
-  g.nrows = item.w & 0xFF;
-  g.n2a = (item.w >> 8) - 64;
-  g.t2a = g.n2a + g.row0 / a.npairs;
-  g.t2b = g.n2a + (g.row0 + g.nrows - 1) / a.npairs;
-  g.bx.row0 = (kXBOfType[item.x] * nx + (g.t2a + N + 1)) * nb;
-  g.bx.len = (g.t2b - g.t2a + 1) * nb;
-  g.bx.lo = g.t2a;
-  g.bc = hblk(a, kr.C, g.s - g.t2b, g.s - g.t2a);
-  g.ba0 = hblk(a, kr.A[0], g.s, g.s);
-  g.ba1 = kr.nmu > 1 ? hblk(a, kr.A[1], g.s, g.s) : HBlk{0, 0, 0};
-  g.sx = 0;
-  g.sc = g.bx.len;
-  g.sa0 = g.sc + g.bc.len;
-  g.sa1 = g.sa0 + g.ba0.len;
+  g.base = item.w;
+  g.alo = ((item.x >> 8) & 0xFF) - 128;
+  g.nrows = item.x >> 16;
+  g.a1 = g.alo + g.row0 / a.npairs;
+  g.a2 = g.alo + (g.row0 + g.nrows - 1) / a.npairs;
+  g.m1 = g.sg - g.a2;
+  g.len = (g.a2 - g.a1 + 1) * nb;
+  const int first = g.w ? a.R.w + 2 * N * nb : (2 * N + 3) * nb;  // the row of index 0
+  g.blk2 = first + g.a1 * nb;
+  g.blk3 = first + g.m1 * nb;
+  g.nfam = g.w ? 1 : a.ncomp;
   return g;
+}
+// family of column group j of an item, and its first row in the wave array; an index outside
+// the record (a family that no component reads at this sg) is clamped into it: its sums are finite
+// and never read
+__device__ __forceinline__ int hfam(const HArgs& a, int4 item, int j) {
+  return a.ncomp == 4 ? j : ((item.x >> 1) & 0x7F) + 2 * j;
+}
+__device__ __forceinline__ int hcol_row(const HArgs& a, int4 item, int j) {
+  const int nb = a.L.nb, N = a.L.N;
+  if (item.x & 1) return a.R.ww - item.y * nb;
+  const int q = hfam(a, item, j);
+  const int m = min(max(basis_col_index(q, item.y), -2 * N - 3), 2 * N - 1);
+  // x G^* = (x^* G)^*, x^* G^* = (x G)^*: the conjugated families read the other array
+  const bool xc = basis_centre_conj(q) != basis_col_conj(q);
+  return (xc ? a.R.xcg : a.R.xg) + (m + 2 * N + 3) * nb;
 }
 
 // packed FP32x2 arithmetic on register pairs (x in the low word)
@@ -275,20 +295,10 @@ __device__ __forceinline__ void split_h2(unsigned long long v, uint32_t& hi, uin
 __device__ __forceinline__ void lds_2x64(uint32_t addr, unsigned long long& a, unsigned long long& b) {
   asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
 }
-__device__ __forceinline__ unsigned long long lds_64(uint32_t addr) {
-  unsigned long long a;
-  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(a) : "r"(addr) : "memory");
-  return a;
-}
-__device__ __forceinline__ void sts_32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
-// The Khatri-Rao values of one row for 8 centres (group h of the thread's 16): x~B at PB, C at
-// PC (shared addresses of the rows in the staged stage, swizzle term folded in: chunk c is at
-// P ^ (c << 4)); CJ: C enters conjugated.  Writes hi / lo words 0..7: four pairs of real parts,
-// then four pairs of imaginary parts.  One 16-byte chunk (four centres) at a time.
-template <bool CJ>
+// The products of one row for 8 centres (group h of the thread's 16): G_a at PB, G_{sg-a} at PC
+// (shared addresses of the rows in the staged stage, swizzle term folded in: chunk c is at
+// P ^ (c << 4)).  Writes hi / lo words 0..7: four pairs of real parts, then four pairs of
+// imaginary parts.  One 16-byte chunk (four centres) at a time.
 __device__ __forceinline__ void kr_group(uint32_t PB, uint32_t PC, int h, uint32_t* hi, uint32_t* lo) {
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
@@ -300,47 +310,60 @@ __device__ __forceinline__ void kr_group(uint32_t PB, uint32_t PC, int h, uint32
     lds_2x64(PC ^ im_off, ci[0], ci[1]);
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-      unsigned long long re, im;
-      if (CJ) {  // x~B conj(C)
-        re = f2fma(xi[p], ci[p], f2mul(xr[p], cr[p]));
-        im = f2sub(f2mul(xi[p], cr[p]), f2mul(xr[p], ci[p]));
-      } else {
-        re = f2sub(f2mul(xr[p], cr[p]), f2mul(xi[p], ci[p]));
-        im = f2fma(xr[p], ci[p], f2mul(xi[p], cr[p]));
-      }
-      split_h2(re, hi[2 * c + p], lo[2 * c + p]);
-      split_h2(im, hi[4 + 2 * c + p], lo[4 + 2 * c + p]);
+      split_h2(f2sub(f2mul(xr[p], cr[p]), f2mul(xi[p], ci[p])), hi[2 * c + p], lo[2 * c + p]);
+      split_h2(f2fma(xr[p], ci[p], f2mul(xi[p], cr[p])), hi[4 + 2 * c + p], lo[4 + 2 * c + p]);
     }
   }
 }
+__device__ __forceinline__ uint4 lds_128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts_128(uint32_t addr, uint4 v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+// CW columns of this thread's TMEM lane
+template <int CW>
+__device__ __forceinline__ void tmem_ld_cols(uint32_t ta, uint32_t* v) {
+  static_assert(CW == 16 || CW == 20 || CW == 24, "columns per quarter");
+  tmem_ld16(ta, v);
+  if (CW == 20) tmem_ld4(ta + 16, v + 16);
+  if (CW == 24) tmem_ld8(ta + 16, v + 16);
+}
 
-// Warp roles: warps 0..15 form the A operand (Khatri-Rao rows, TMEM) and the B operand
-// (shared memory) of each stage; warp 16 issues the MMAs (one thread); warp 17 stages each
-// stage's rows of the wave array with TMA (one thread).  Rings and their mbarriers (counts in
-// brackets):
-//   staged input  in_full [1 + TMA bytes] / in_empty [16 producer warps]
-//   A and B       ab_full [16 producer warps] / ab_empty [1, tcgen05.commit]
+// Warp roles: warps 0..15 form the A operand (row products, TMEM); warps 16 and 17 the B operand
+// (shared memory) of each stage; warp 18 issues the MMAs (one thread); warp 19 stages each
+// stage's rows of the wave array with bulk copies (one thread).  Rings and their mbarriers
+// (counts in brackets):
+//   staged input  in_full [1 + copied bytes] / in_empty [18 forming warps]
+//   A and B       ab_full [18 forming warps] / ab_empty [1, tcgen05.commit]
 //   partial sums  dfull [1, tcgen05.commit] / dempty [16 producer warps]
+// CW: D columns per producer quarter (4 CW in all); SLOTS: A/B ring depth, what the
+// 512 TMEM columns leave next to two D buffers.
+template <int CW, int SLOTS>
 __global__ void __launch_bounds__(kHThreads, 1)
 contract_h16_kernel(const __grid_constant__ HArgs args) {
+  constexpr int kDStride = CW == 16 ? 64 : 96, kABase = 2 * kDStride;
+  static_assert(4 * CW <= kDStride && kABase + SLOTS * kHACols <= (int)kHTmemCols, "TMEM columns");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = smem_raw + ((1024 - (saddr(smem_raw) & 1023)) & 1023);
   const Layout L = args.L;
-  const int nb = L.nb, N = L.N, npairs = args.npairs;
+  const int nb = L.nb, npairs = args.npairs;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t atom_bytes = (uint32_t)args.npad_max * 128u;  // one 128-byte-wide K-atom of a B tile
   const uint32_t bslot_bytes = 4u * atom_bytes;                  // hi tile (2 atoms) | lo tile (2 atoms)
   const uint32_t in_bytes = (uint32_t)args.stage_rows * 512u;    // one staged stage: rows of 512 bytes
   const int S_in = args.in_stages;
-  unsigned char* in_base = sm + kHSlots * bslot_bytes;
+  unsigned char* in_base = sm + SLOTS * bslot_bytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(in_base + (size_t)S_in * in_bytes);
   uint64_t* in_full = bars;
   uint64_t* in_empty = in_full + kHMaxIn;
   uint64_t* ab_full = in_empty + kHMaxIn;
-  uint64_t* ab_empty = ab_full + kHSlots;
-  uint64_t* dfull = ab_empty + kHSlots;  // [2]
-  uint64_t* dempty = dfull + 2;          // [2]
-  uint64_t* drain = dempty + 2;          // [1]
+  uint64_t* ab_empty = ab_full + kHMaxSlots;
+  uint64_t* dfull = ab_empty + kHMaxSlots;  // [2]
+  uint64_t* dempty = dfull + 2;             // [2]
+  uint64_t* drain = dempty + 2;             // [1]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -353,10 +376,10 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
   if (tid == 32) {
     for (int k = 0; k < S_in; ++k) {
       mbar_init(&in_full[k], 1);
-      mbar_init(&in_empty[k], kHProducerWarps);
+      mbar_init(&in_empty[k], kHArrivals);
     }
-    for (int k = 0; k < kHSlots; ++k) {
-      mbar_init(&ab_full[k], kHProducerWarps);
+    for (int k = 0; k < SLOTS; ++k) {
+      mbar_init(&ab_full[k], kHArrivals);
       mbar_init(&ab_empty[k], 1);
     }
     for (int k = 0; k < 2; ++k) {
@@ -395,97 +418,53 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
   if (warp < kHProducerWarps) {
     // ---------------------------------------------------------------------- producers
     const int grp = warp & 3, qq = warp >> 2;  // TMEM lane group; 16-centre quarter of a stage
-    const uint32_t in_addr = saddr(in_base), b_addr = saddr(sm);
+    const uint32_t in_addr = saddr(in_base);
     int islot = 0, aslot = 0;
     uint32_t iph = 0, aph = 0;
     long long gs = 0;  // partial sums (stages) so far
     for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
       const int4 item = args.items[it];
-      const KRType kr = kKR[item.x];
-      const HGeo g = hgeo(args, item, kr);
-      const int nmu = kr.nmu, ncols = 2 * nmu * nb, nv = nmu * nb;
-      const int npad = (ncols + 15) & ~15;
+      const HGeo g = hgeo(args, item);
+      const int ncols = 2 * g.nfam * nb, npad = (ncols + 15) & ~15;
       const int rl = grp * 32 + lane;  // tile row = TMEM lane
       const bool row_ok = rl < g.nrows;
       const int rr = g.row0 + (row_ok ? rl : 0);
-      const int n2 = g.n2a + rr / npairs, n3 = g.s - n2;
+      const int av = g.alo + rr / npairs;
       int b2, b3;
-      pair_of(rr % npairs, nb, b2, b3);
-      const int eB = g.sx + (n2 - g.t2a) * nb + b2;
-      const int eC = g.sc + hblk_index(g.bc, kr.C, n3, b3, nb);
-      const bool cjC = kr.C.conj != 0;
-      // this row's x~B and C rows, quarter qq, in a staged stage, with the swizzle term of their
+      basis_pair(rr % npairs, nb, b2, b3);
+      // this row's two factors, quarter qq, in a staged stage, with the swizzle term of their
       // rows in the wave array folded in (chunk c at P ^ (c << 4))
-      const int rB = g.bx.row0 + (eB - g.sx), rC = g.bc.row0 + (eC - g.sc);
-      const uint32_t xB0 = (uint32_t)eB * 512u + qq * 128u + ((uint32_t)(rB & 7) << 4);
-      const uint32_t xC0 = (uint32_t)eC * 512u + qq * 128u + ((uint32_t)(rC & 7) << 4);
-      // the B columns this warp forms: column pairs v = warp, warp + 16 (component slot v / nb,
-      // Th1 = v % nb); lane = centres 2 lane, 2 lane + 1 of the stage
-      // shared offsets: aoff = the lane's two real parts of A (the imaginary parts: chunk + 4,
-      // i.e. ^ 64); boff[o] = the real-part K word of output o (0: real, 1: imaginary) in the
-      // hi tile (the imaginary-part K word: the next chunk, i.e. ^ 16)
-      uint32_t aoff[2], boff[2][2], msk[2];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int v = warp + j * kHProducerWarps;
-        int eA = 0, rA = 0;
-        bool cj = false;
-        if (v < nv) {
-          const int b1 = v % nb;
-          if (v < nb) {
-            eA = g.sa0 + hblk_index(g.ba0, kr.A[0], g.s, b1, nb);
-            rA = g.ba0.row0 + (eA - g.sa0);
-            cj = kr.A[0].conj != 0;
-          } else {
-            eA = g.sa1 + hblk_index(g.ba1, kr.A[1], g.s, b1, nb);
-            rA = g.ba1.row0 + (eA - g.sa1);
-            cj = kr.A[1].conj != 0;
-          }
-        }
-        aoff[j] = (uint32_t)eA * 512u + (uint32_t)(lane >> 3) * 128u + (lane & 1) * 8 +
-                  ((uint32_t)(((lane & 7) >> 1) ^ (rA & 7)) << 4);
-        // real output: K_re <- A_r, K_im <- -A_i (conj A: +A_i); imaginary output: K_re <- A_i
-        // (conj: -A_i), K_im <- A_r
-        msk[j] = cj ? 0u : 0x80008000u;
-        const int q = lane >> 2;                       // MMA group of the lane's centres
-        const uint32_t atom = (uint32_t)(q >> 2) * atom_bytes, within = (lane & 3) * 4;
-        const int ch = 2 * (q & 3);
-#pragma unroll
-        for (int o = 0; o < 2; ++o) {
-          const int n = 2 * v + o;
-          boff[j][o] = atom + (uint32_t)(n >> 3) * 1024u + (uint32_t)(n & 7) * 128u + within +
-                       ((uint32_t)(ch ^ (n & 7)) << 4);
-        }
-      }
-      float accD[16];  // FP32 sums of the promoted partials: this row, 16 columns
-      const bool has_cols = qq * 16 < npad;
+      const int e2 = (av - g.a1) * nb + b2, e3 = (g.sg - av - g.m1) * nb + b3;
+      const int r2 = g.blk2 + e2, r3 = g.blk3 + e3;
+      const uint32_t x2 = (uint32_t)e2 * 512u + qq * 128u + ((uint32_t)(r2 & 7) << 4);
+      const uint32_t x3 = (uint32_t)(g.len + e3) * 512u + qq * 128u + ((uint32_t)(r3 & 7) << 4);
+      float accD[CW];  // FP32 sums of the promoted partials: this row, CW columns
+      const bool has_cols = qq * CW < npad;
       // Software pipeline over the stages (k = this stage):
-      //  * the partial sum of stage k - 2 is read out of TMEM at the end of this stage
-      //    (tcgen05.ld issued there, waited for after the first half of the next stage's rows),
-      //    then its D buffer is released, before the MMAs of stage k are signalled;
+      //  * the partial sum of stage k - 2 is taken out of TMEM at the start of this stage: its MMAs
+      //    were signalled in the middle of stage k - 1;
       //  * the rows of stage k - 1 were stored into TMEM at the end of the previous iteration;
       //    their completion is awaited (and the MMA warp signalled) only after the first half
       //    of this stage's rows is formed, so the store latency is hidden behind that work.
-      // The MMAs of stage k - 1 thus start one iteration late, which the three A/B slots absorb.
-      auto promote_issue = [&](long long gg, uint32_t* v) {
+      // The MMAs of stage k - 1 thus start one iteration late; the wait for the slot of stage k
+      // comes after the first half of its rows, when the MMAs of stage k - SLOTS are done.
+      auto promote = [&](long long gg) {
         const int buf = (int)(gg & 1);
         wait(&dfull[buf], (uint32_t)((gg >> 1) & 1));
         tc_fence_after();
-        if (has_cols) tmem_ld16(tmem + ((uint32_t)(grp * 32) << 16) + buf * 64 + qq * 16, v);
-      };
-      auto promote_finish = [&](long long gg, const uint32_t* v) {
         if (has_cols) {
+          uint32_t v[CW];
+          tmem_ld_cols<CW>(tmem + ((uint32_t)(grp * 32) << 16) + buf * kDStride + qq * CW, v);
           tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 16; ++j) accD[j] += __uint_as_float(v[j]);
+          for (int j = 0; j < CW; ++j) accD[j] += __uint_as_float(v[j]);
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&dempty[(int)(gg & 1)]);
+        if (lane == 0) mbar_arrive(&dempty[buf]);
       };
-      auto publish = [&](int slot) {  // the rows (TMEM) and columns (shared) of a slot are complete
+      auto publish = [&](int slot) {  // the rows (TMEM) of a slot are complete
         tmem_wait_st();
-        fence_async_smem();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&ab_full[slot]);
@@ -499,93 +478,125 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
       for (; si < args.plan.nseg && args.plan.seg[si].slot == slot; ++si)
         nstage += (seg_live(args.plan.seg[si]) + kHCentres - 1) / kHCentres;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) accD[j] = 0.f;
+      for (int j = 0; j < CW; ++j) accD[j] = 0.f;
       int prev_slot = 0;
-      uint32_t pv[16];  // a partial sum on its way out of TMEM: read at the end of one stage,
-                        // added in the middle of the next
       for (int k = 0; k < nstage; ++k) {
+        if (k >= 2) promote(gs + k - 2);
         wait(&in_full[islot], iph);
-        wait(&ab_empty[aslot], aph ^ 1u);
-        tc_fence_after();
         const uint32_t st = in_addr + (uint32_t)islot * in_bytes;
-        const uint32_t bt = b_addr + (uint32_t)aslot * bslot_bytes;
-        // B operand: the real embedding of A(Th1), fp16 hi and lo tiles
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          if (warp + j * kHProducerWarps >= nv) break;
-          uint32_t arh, arl, aih, ail;
-          split_h2(lds_64(st + aoff[j]), arh, arl);
-          split_h2(lds_64(st + (aoff[j] ^ 64u)), aih, ail);
-          const uint32_t m1 = msk[j], m2 = msk[j] ^ 0x80008000u;
-          const uint32_t r0 = bt + boff[j][0], r1 = bt + boff[j][1], lt = 2 * atom_bytes;
-          sts_32(r0, arh);
-          sts_32(r0 ^ 16u, aih ^ m1);
-          sts_32(r1, aih ^ m2);
-          sts_32(r1 ^ 16u, arh);
-          sts_32(r0 + lt, arl);
-          sts_32((r0 ^ 16u) + lt, ail ^ m1);
-          sts_32(r1 + lt, ail ^ m2);
-          sts_32((r1 ^ 16u) + lt, arl);
-        }
-        // A operand (TMEM): this row's Khatri-Rao values for the warp's 16 centres, in two
-        // groups of 8; the previous stage is published between them
-        const uint32_t PB = st + xB0, PC = st + xC0;
-        const uint32_t acol = tmem + ((uint32_t)(grp * 32) << 16) + kHDCols + aslot * kHACols + qq * 16;
+        // A operand (TMEM): this row's products for the warp's 16 centres, in two groups of 8;
+        // the previous stage is published between them
+        const uint32_t PB = st + x2, PC = st + x3;
+        const uint32_t acol = tmem + ((uint32_t)(grp * 32) << 16) + kABase + aslot * kHACols + qq * 16;
         {
           uint32_t hi[8], lo[8];
-          if (cjC) kr_group<true>(PB, PC, 0, hi, lo);
-          else kr_group<false>(PB, PC, 0, hi, lo);
-          if (k >= 3) promote_finish(gs + k - 3, pv);
+          kr_group(PB, PC, 0, hi, lo);
           if (k >= 1) publish(prev_slot);
+          wait(&ab_empty[aslot], aph ^ 1u);
+          tc_fence_after();
           tmem_st8(acol, hi);
           tmem_st8(acol + 64, lo);
         }
         {
           uint32_t hi[8], lo[8];
-          if (cjC) kr_group<true>(PB, PC, 1, hi, lo);
-          else kr_group<false>(PB, PC, 1, hi, lo);
+          kr_group(PB, PC, 1, hi, lo);
           // every value this warp loaded from the staged stage has been used: it can be refilled
           __syncwarp();
           if (lane == 0) mbar_arrive(&in_empty[islot]);
           tmem_st8(acol + 8, hi);
           tmem_st8(acol + 64 + 8, lo);
         }
-        if (k >= 2) promote_issue(gs + k - 2, pv);
         prev_slot = aslot;
         if (++islot == S_in) { islot = 0; iph ^= 1u; }
-        if (++aslot == kHSlots) { aslot = 0; aph ^= 1u; }
+        if (++aslot == SLOTS) { aslot = 0; aph ^= 1u; }
       }
-      // drain the pipeline: the partial sum read at the end of the last stage, the last
-      // stage's rows, then the last two partial sums
-      if (nstage >= 3) promote_finish(gs + nstage - 3, pv);
+      // drain the pipeline: the last stage's rows, then the last two partial sums
       if (nstage >= 1) publish(prev_slot);
-      for (long long gg = gs + (nstage >= 2 ? nstage - 2 : 0); gg < gs + nstage; ++gg) {
-        promote_issue(gg, pv);
-        promote_finish(gg, pv);
-      }
+      for (long long gg = gs + (nstage >= 2 ? nstage - 2 : 0); gg < gs + nstage; ++gg) promote(gg);
       gs += nstage;
       // ---------------------------------------------------------------- epilogue
       if (row_ok && has_cols && nstage > 0) {  // (an empty run adds nothing)
-        const int pr = rr % npairs, nx = 2 * N + 3;
-        const int kx = h_scale_exp(args.rowmax[g.bx.row0 + (eB - g.sx)]);
-        const int kc = h_scale_exp(args.rowmax[g.bc.row0 + (eC - g.sc)]);
+        const int kr = h_scale_exp(args.rowmax[r2]) + h_scale_exp(args.rowmax[r3]);
+        const size_t row = (size_t)g.base + (av - g.alo), pr = rr % npairs;
+        double2* out = args.red + (size_t)slot * args.red_stride;
+        out += g.w ? args.red_w + row * nb * npairs + pr : row * 4 * nb * npairs + pr;
 #pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-          const int n = qq * 16 + j;
-          if (n < ncols) {
-            const int ga = n / (2 * nb), b1 = (n >> 1) % nb;
-            const int mu = ga ? kr.mu[1] : kr.mu[0];
-            const int arow = ga ? g.ba1.row0 + hblk_index(g.ba1, kr.A[1], g.s, b1, nb)
-                                : g.ba0.row0 + hblk_index(g.ba0, kr.A[0], g.s, b1, nb);
-            const double unscale = h_pow2d(-(kx + kc + h_scale_exp(args.rowmax[arow])));
-            const size_t o = ((((size_t)mu * nx + (n2 + N + 1)) * nx + (n3 + N + 1)) * nb + b1) * npairs + pr;
-            double* p = args.red + (size_t)slot * args.red_stride + 2 * o;
-            p[0] += (double)accD[j] * unscale;
-            p[1] += (double)accD[j + 1] * unscale;
+        for (int j = 0; j < CW; j += 2) {
+          const int v = (qq * CW + j) >> 1;
+          if (2 * v < ncols) {
+            const int f = v / nb, b1 = v - f * nb;
+            const double unscale = h_pow2d(-(kr + h_scale_exp(args.rowmax[hcol_row(args, item, f) + b1])));
+            double2* p = out + (size_t)(g.w ? b1 : hfam(args, item, f) * nb + b1) * npairs;
+            double2 d = *p;
+            d.x += (double)accD[j] * unscale;
+            d.y += (double)accD[j + 1] * unscale;
+            *p = d;
           }
         }
       }
       }  // runs of segments
+    }
+  } else if (warp < kHWarpMma) {
+    // ---------------------------------------------------------------------- B operand
+    // The real embedding of the columns, fp16 hi and lo tiles: for column value A = (A_r, A_i)
+    // tile row 2 v (real output) holds A_r at the real and -A_i at the imaginary K, row 2 v + 1
+    // (imaginary output) A_i and A_r; a conjugated column has A_i of the other sign.  A lane takes
+    // 8 centres (one 16-byte chunk each of A_r and A_i, hi and lo) of column pair v: eight
+    // 16-byte stores, the lanes of the upper K-atom taking A_r and A_i in the other order, so that
+    // the eight lanes of a phase hit eight different bank groups.
+    const uint32_t in_addr = saddr(in_base), b_addr = saddr(sm);
+    int islot = 0, aslot = 0;
+    uint32_t iph = 0, aph = 0;
+    for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
+      const int4 item = args.items[it];
+      const HGeo g = hgeo(args, item);
+      // lane: centre chunk q of column pairs v0, v0 + 8, ...
+      const int t0 = (warp - kHProducerWarps) * 32 + lane, v0 = t0 >> 3, q = t0 & 7;
+      const int npair = g.nfam * nb;
+      const bool up = q >= 4;  // upper K-atom
+      const uint32_t src0 = (uint32_t)(2 * g.len + v0) * 512u + q * 16u + (up ? 128u : 0u);
+      const uint32_t n7 = (2u * v0) & 7u;
+      const uint32_t dst0 = (uint32_t)(q >> 2) * atom_bytes + ((2u * v0) >> 3) * 1024u + n7 * 128u +
+                            (((uint32_t)(2 * (q & 3)) ^ n7) << 4) + (up ? 16u : 0u);
+      // (n7 is even: the row below differs in the lowest chunk bit and the row only)
+      const uint32_t dst1 = (uint32_t)(q >> 2) * atom_bytes + ((2u * v0) >> 3) * 1024u + (n7 + 1u) * 128u +
+                            ((((uint32_t)(2 * (q & 3)) ^ (n7 + 1u)) << 4) ^ (up ? 16u : 0u));
+      uint32_t conj = 0;  // bit i: column pair v0 + 8 i belongs to a conjugated family
+      for (int v = v0, i = 0; v < npair; v += 8, ++i)
+        if (!g.w && basis_col_conj(hfam(args, item, v / nb))) conj |= 1u << i;
+      for (int si = 0; si < args.plan.nseg; ++si) {
+        const int nstage = (seg_live(args.plan.seg[si]) + kHCentres - 1) / kHCentres;
+        for (int k = 0; k < nstage; ++k) {
+          wait(&in_full[islot], iph);
+          wait(&ab_empty[aslot], aph ^ 1u);
+          uint32_t src = in_addr + (uint32_t)islot * in_bytes + src0;
+          uint32_t d = b_addr + (uint32_t)aslot * bslot_bytes;
+          uint32_t cbits = conj;
+          for (int v = v0; v < npair; v += 8, src += 8 * 512u, d += 2048u, cbits >>= 1) {
+            // sign of the imaginary part in row 2 v; row 2 v + 1 has the other one
+            const uint32_t s0 = cbits & 1u ? 0u : 0x80008000u, s1 = s0 ^ 0x80008000u;
+            const uint32_t mx0 = up ? s0 : 0u, my0 = up ? 0u : s0, mx1 = up ? s1 : 0u, my1 = up ? 0u : s1;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {  // hi, lo
+              // x: the real part (lower K-atom) or the imaginary part (upper), y: the other
+              const uint4 x = lds_128(src + h * 256u), y = lds_128((src ^ 128u) + h * 256u);
+              const uint32_t e = d + dst0 + h * 2u * atom_bytes, f = d + dst1 + h * 2u * atom_bytes;
+              sts_128(e, make_uint4(x.x ^ mx0, x.y ^ mx0, x.z ^ mx0, x.w ^ mx0));
+              sts_128(e ^ 16u, make_uint4(y.x ^ my0, y.y ^ my0, y.z ^ my0, y.w ^ my0));
+              sts_128(f, make_uint4(y.x ^ my1, y.y ^ my1, y.z ^ my1, y.w ^ my1));
+              sts_128(f ^ 16u, make_uint4(x.x ^ mx1, x.y ^ mx1, x.z ^ mx1, x.w ^ mx1));
+            }
+          }
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(&in_empty[islot]);
+            mbar_arrive(&ab_full[aslot]);
+          }
+          if (++islot == S_in) { islot = 0; iph ^= 1u; }
+          if (++aslot == SLOTS) { aslot = 0; aph ^= 1u; }
+        }
+      }
     }
   } else if (warp == kHWarpMma) {
     // ---------------------------------------------------------------------- MMA issuer
@@ -595,8 +606,8 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
       uint32_t aph = 0;
       long long gs = 0;
       for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
-        const KRType kr = kKR[args.items[it].x];
-        const int npad = (2 * kr.nmu * nb + 15) / 16 * 16;
+        const HGeo g = hgeo(args, args.items[it]);
+        const int npad = (2 * g.nfam * nb + 15) / 16 * 16;
         const uint32_t id = idesc(0u, npad);  // fp16 A and B, FP32 D
         for (int si = 0; si < args.plan.nseg; ++si) {
         const int nstage = (seg_live(args.plan.seg[si]) + kHCentres - 1) / kHCentres;
@@ -605,22 +616,28 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
           if (gs >= 2) wait(&dempty[buf], (uint32_t)(((gs >> 1) - 1) & 1));
           wait(&ab_full[aslot], aph);
           tc_fence_after();
-          const uint32_t d = tmem + buf * 64;
-          const uint32_t ah = tmem + kHDCols + aslot * kHACols, al = ah + 64;
+          const uint32_t d = tmem + buf * kDStride;
+          const uint32_t ah = tmem + kABase + aslot * kHACols, al = ah + 64;
           // descriptor of the slot's hi tile: start-address field (address / 16) plus the
           // offset / 16 (no carry: shared addresses stay below 2^18)
           const uint64_t db = dbase + (uint64_t)((aslot * bslot_bytes) >> 4);
           const uint64_t dl = (uint64_t)((2 * atom_bytes) >> 4);
+          // the two small terms of every K step first, while the sum is small: the unit cuts each
+          // addition to the sum's last bit, so the order leaves 8 such cuts at full size, not 24
 #pragma unroll
           for (int q = 0; q < 8; ++q) {  // K = 16 halves = 8 centres per MMA
             const uint64_t bh = db + (uint64_t)((((q >> 2) * atom_bytes) + (q & 3) * 32) >> 4);
-            mma_f16(d, ah + q * 8, bh, id, q > 0 ? 1u : 0u);
-            mma_f16(d, ah + q * 8, bh + dl, id, 1u);
+            mma_f16(d, ah + q * 8, bh + dl, id, q > 0 ? 1u : 0u);
             mma_f16(d, al + q * 8, bh, id, 1u);
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const uint64_t bh = db + (uint64_t)((((q >> 2) * atom_bytes) + (q & 3) * 32) >> 4);
+            mma_f16(d, ah + q * 8, bh, id, 1u);
           }
           mma_commit(&ab_empty[aslot]);
           mma_commit(&dfull[buf]);
-          if (++aslot == kHSlots) { aslot = 0; aph ^= 1u; }
+          if (++aslot == SLOTS) { aslot = 0; aph ^= 1u; }
         }
         }  // segments
       }
@@ -630,9 +647,9 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
       if (!mbar_wait(drain, 0u, 4000000000LL)) err = 1;
     }
     __syncwarp();
-  } else if (warp == kHWarpLoad) {
+  } else {
     // ---------------------------------------------------------------------- bulk-copy loader
-    // One thread: per stage the four blocks of the item, each a contiguous range of the
+    // One thread: per stage the blocks of the item, each a contiguous range of the
     // stage-major wave array, copied with one cp.async.bulk each.
     if (lane == 0) {
       int islot = 0;
@@ -640,18 +657,22 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
       int last[kHMaxIn];  // parity of the last phase issued per slot (-1: none)
       for (int k = 0; k < kHMaxIn; ++k) last[k] = -1;
       for (int it = blockIdx.x; it < args.n_items; it += gridDim.x) {
-        const KRType kr = kKR[args.items[it].x];
-        const HGeo g = hgeo(args, args.items[it], kr);
-        const HBlk blk[4] = {g.bx, g.bc, g.ba0, g.ba1};
-        const int srow[4] = {g.sx, g.sc, g.sa0, g.sa1};
-        bool ok = g.sa1 + g.ba1.len <= args.stage_rows;
-        for (int b = 0; b < 4; ++b)
-          ok = ok && (blk[b].len == 0 || (blk[b].row0 >= 0 && blk[b].row0 + blk[b].len <= args.rows));
+        const int4 item = args.items[it];
+        const HGeo g = hgeo(args, item);
+        int blk[6], n = 2 + g.nfam;
+        blk[0] = g.blk2;
+        blk[1] = g.blk3;
+        for (int j = 0; j < g.nfam; ++j) blk[2 + j] = hcol_row(args, item, j);
+        const int rows = 2 * g.len + g.nfam * nb;
+        bool ok = rows <= args.stage_rows;
+        for (int b = 0; b < n; ++b) {
+          const int len = b < 2 ? g.len : nb;
+          ok = ok && blk[b] >= 0 && blk[b] + len <= args.R.rows;
+        }
         if (!ok) {  // never for the supported shapes
           *abort_flag = 1;
           err = 1;
         }
-        const uint32_t bytes = (uint32_t)(g.sa1 + g.ba1.len) * 512u;
         for (int si = 0; si < args.plan.nseg; ++si) {
         const WaveSeg& sgm = args.plan.seg[si];
         const int nstage = (seg_live(sgm) + kHCentres - 1) / kHCentres, kst0 = sgm.off / kHCentres;
@@ -659,14 +680,14 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
           wait(&in_empty[islot], iph ^ 1u);
           if (!*abort_flag) {  // nothing more is copied once the CTA gives up
             last[islot] = (int)iph;
-            mbar_expect_tx(&in_full[islot], bytes);
+            mbar_expect_tx(&in_full[islot], (uint32_t)rows * 512u);
             unsigned char* st = in_base + (size_t)islot * in_bytes;
-            const float* src = args.wave + (size_t)(kst0 + k) * args.rows * 128;
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-              if (blk[b].len > 0)
-                bulk_load(st + srow[b] * 512, src + (size_t)blk[b].row0 * 128, (uint32_t)blk[b].len * 512u,
-                          &in_full[islot]);
+            const float* src = args.wave + (size_t)(kst0 + k) * args.R.rows * 128;
+            for (int b = 0; b < n; ++b) {
+              const int len = b < 2 ? g.len : nb;
+              bulk_load(st, src + (size_t)blk[b] * 128, (uint32_t)len * 512u, &in_full[islot]);
+              st += len * 512;
+            }
           }
           if (++islot == S_in) { islot = 0; iph ^= 1u; }
         }
@@ -687,78 +708,107 @@ contract_h16_kernel(const __grid_constant__ HArgs args) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kHTmemCols) : "memory");
 }
 
-// rows per staged stage: the x~B and C blocks of at most the tile's n2 values (128 rows =
-// 128 / pairs values of n2, +2 for misalignment, at most 2N + 3) and two A blocks
-int h_stage_rows(int nb, int N) {
-  int rows = 128 / (nb * (nb + 1) / 2) + 2;
-  if (rows > 2 * N + 3) rows = 2 * N + 3;
-  return 2 * rows * nb + 2 * nb;
+// families per X item: four while their columns fit a D buffer of 96, two in two groups beyond
+int h_ncomp(int nb) { return nb <= 12 ? 4 : 2; }
+int h_npad_max(int nb) { return (2 * h_ncomp(nb) * nb + 15) / 16 * 16; }
+// D columns per producer quarter and A/B slots next to the two D buffers
+int h_cw(int nb) { return h_npad_max(nb) <= 64 ? 16 : h_npad_max(nb) <= 80 ? 20 : 24; }
+int h_slots(int nb) { return h_cw(nb) == 16 ? 3 : 2; }
+// rows per tile: one TMEM lane each; half of them for a single bin, whose rows all have an a of
+// their own (staged blocks of 128 rows each would not fit twice)
+int h_tile_rows(int nb) { return nb == 1 ? 64 : 128; }
+// rows per staged stage: two blocks of at most the tile's a values (+2 where tiles cut through
+// the pairs of an a) and the column rows
+int h_stage_rows(int nb) {
+  const int np = nb * (nb + 1) / 2;
+  const int av = np == 1 ? h_tile_rows(nb) : h_tile_rows(nb) / np + 2;
+  return 2 * av * nb + h_ncomp(nb) * nb;
 }
-int h_npad_max(int nb) { return (4 * nb + 15) / 16 * 16; }
-size_t h_fixed_smem(int nb) { return (size_t)kHSlots * 4 * h_npad_max(nb) * 128 + 1024 + 512; }
-int h_in_stages(int nb, int N) {
-  const size_t per = (size_t)h_stage_rows(nb, N) * 512;
+size_t h_fixed_smem(int nb) { return (size_t)h_slots(nb) * 4 * h_npad_max(nb) * 128 + 1024 + 512; }
+int h_in_stages(int nb) {
+  const size_t per = (size_t)h_stage_rows(nb) * 512;
   const size_t room = 227 * 1024 - h_fixed_smem(nb);
   int k = (int)(room / per);
   if (k > kHMaxIn) k = kHMaxIn;
   return k >= 2 ? k : 0;
 }
-size_t h_smem_bytes(int nb, int N) {
-  return h_fixed_smem(nb) + (size_t)h_in_stages(nb, N) * h_stage_rows(nb, N) * 512;
+size_t h_smem_bytes(int nb) { return h_fixed_smem(nb) + (size_t)h_in_stages(nb) * h_stage_rows(nb) * 512; }
+
+template <int CW, int SLOTS>
+cudaError_t launch_h16(const HArgs& a, int sms, size_t smem, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(contract_h16_kernel<CW, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  contract_h16_kernel<CW, SLOTS><<<sms, kHThreads, smem, s>>>(a);
+  ++g_launches;
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-int h16_wave_rows(const Layout& L) { return (kXBTypes * (2 * L.N + 3) + L.nG + 4 * L.N + 1) * L.nb; }
+int h16_wave_rows(const Layout& L) { return HRows::make(L).rows; }
 static int h16_wave_pitch(int T) { return (T + kHCentres - 1) / kHCentres * kHCentres; }
 
-bool h16_supported(const Layout& L) {
-  return L.nb >= 1 && 4 * L.nb <= 64 && h_in_stages(L.nb, L.N) >= 2;
-}
+bool h16_supported(const Layout& L) { return L.nb >= 1 && L.nb <= 16 && h_in_stages(L.nb) >= 2; }
 size_t contract_h16_wave_bytes(const Layout& L, int T) {
   return (size_t)h16_wave_rows(L) * h16_wave_pitch(T) * sizeof(float2);
 }
 size_t contract_h16_rowmax_bytes(const Layout& L) { return (size_t)h16_wave_rows(L) * sizeof(unsigned); }
 
-cudaError_t contract_wave_h16(const Layout& L, const float2* rec, const float2* xw, const WavePlan& plan,
-                              double* red, const int4* items, int n_items, float2* wave, unsigned* rowmax,
-                              int* status, long long timeout, cudaStream_t s) {
+// work items: tiles of the rows of one sg (a by a, the pairs of an a side by side)
+void h16_build_items(const Basis& B, std::vector<int4>& items) {
+  items.clear();
+  const int tile = h_tile_rows(B.nb), groups = 4 / h_ncomp(B.nb);
+  for (int g = 0; g < groups; ++g)
+    for (int q = 0; q < B.nsg; ++q) {
+      const int rows = B.xlen[q] * B.npairs;
+      for (int r = 0; r < rows; r += tile)
+        items.push_back(make_int4((g << 1) | ((B.xlo[q] + 128) << 8) | (std::min(tile, rows - r) << 16), B.sg0 + q, r,
+                                  B.xbase[q]));
+    }
+  for (int t = 0; t <= 2 * B.N; ++t) {
+    const int rows = B.wlen(t) * B.npairs;
+    for (int r = 0; r < rows; r += tile)
+      items.push_back(make_int4(1 | ((128 - B.N) << 8) | (std::min(tile, rows - r) << 16), -t, r, B.wbase(t)));
+  }
+}
+
+cudaError_t contract_wave_h16(const Layout& L, const Basis& B, const float2* rec, const float2* xw,
+                              const WavePlan& plan, double* red, const int4* items, int n_items, float2* wave,
+                              unsigned* rowmax, int* status, long long timeout, cudaStream_t s) {
   if (plan.total <= 0 || plan.nseg <= 0) return cudaSuccess;
   for (int i = 0; i < plan.nseg; ++i)  // segments start at stage boundaries
     if (plan.seg[i].off % kHCentres != 0) return cudaErrorInvalidValue;
-  const int rows = h16_wave_rows(L), pitch = h16_wave_pitch(plan.total);
-  const int row_g = kXBTypes * (2 * L.N + 3) * L.nb, row_w = row_g + L.nG * L.nb;
+  const HRows R = HRows::make(L);
+  const int rows = R.rows, pitch = h16_wave_pitch(plan.total);
   cudaError_t e = cudaMemsetAsync(rowmax, 0, (size_t)rows * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
-  hwave_rowmax_kernel<<<dim3((rows + 31) / 32, (plan.total + 127) / 128), 256, 0, s>>>(L, rec, xw, plan, row_g,
-                                                                                     row_w, rows, rowmax);
-  hwave_transpose_kernel<<<dim3((rows + 31) / 32, pitch / 32), 256, 0, s>>>(
-      L, rec, xw, plan, row_g, row_w, rows, rowmax, reinterpret_cast<float*>(wave));
+  hwave_rowmax_kernel<<<dim3((rows + 31) / 32, (plan.total + 127) / 128), 256, 0, s>>>(L, rec, xw, plan, R, rowmax);
+  hwave_transpose_kernel<<<dim3((rows + 31) / 32, pitch / 32), 256, 0, s>>>(L, rec, xw, plan, R, rowmax,
+                                                                          reinterpret_cast<float*>(wave));
   g_launches += 2;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   HArgs a;
-  a.L = L; a.plan = plan; a.red = red; a.red_stride = tc_reduced_doubles(L);
-  a.npairs = L.nb * (L.nb + 1) / 2;
+  a.L = L; a.R = R; a.plan = plan;
+  a.red = reinterpret_cast<double2*>(red); a.red_stride = B.elems(); a.red_w = B.woff();
+  a.npairs = B.npairs;
   a.items = items; a.n_items = n_items;
-  a.row_g = row_g; a.row_w = row_w;
+  a.ncomp = h_ncomp(L.nb);
   a.rowmax = rowmax;
   a.wave = reinterpret_cast<const float*>(wave);
-  a.rows = rows;
-  a.in_stages = h_in_stages(L.nb, L.N);
-  a.stage_rows = h_stage_rows(L.nb, L.N);
+  a.in_stages = h_in_stages(L.nb);
+  a.stage_rows = h_stage_rows(L.nb);
   a.npad_max = h_npad_max(L.nb);
   a.timeout = timeout; a.status = status;
   if (a.in_stages < 2) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const size_t smem = h_smem_bytes(L.nb, L.N);
-  e = cudaFuncSetAttribute(contract_h16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  contract_h16_kernel<<<sms, kHThreads, smem, s>>>(a);
-  ++g_launches;
-  return cudaGetLastError();
+  const size_t smem = h_smem_bytes(L.nb);
+  if (h_cw(L.nb) == 16) return launch_h16<16, 3>(a, sms, smem, s);
+  if (h_cw(L.nb) == 20) return launch_h16<20, 2>(a, sms, smem, s);
+  return launch_h16<24, 2>(a, sms, smem, s);
 }
 
 }  // namespace ext4pcf

@@ -21,8 +21,9 @@ def _case(nb, seed=31, n=150):
     return pos, rng.normal(0, 0.3, pos.shape), rng.uniform(0.5, 1.5, n), np.geomspace(0.5, 7.0, nb + 1)
 
 
-@pytest.mark.parametrize("prec,nb,nmax", [(p, nb, N) for p in ("fp64", "fp32") for nb, N in
-                                          SHAPES + [(17, 1), (24, 0), (25, 1), (32, 1)]])
+@pytest.mark.parametrize("prec,nb,nmax", [(p, nb, N) for p in ("fp64", "fp32", "f16x3") for nb, N in
+                                          SHAPES + ([] if p == "f16x3" else [(17, 1), (24, 0), (25, 1), (32, 1)])
+                                          + ([(2, 9), (6, 4), (10, 5), (14, 2), (15, 1)] if p == "f16x3" else [])])
 def test_matches_oracle(torch_cuda, oracle, prec, nb, nmax):  # noqa: F811
     pos, sh, w, edges = _case(nb)
     ref = oracle.measure(pos, sh, w, edges, nmax)
@@ -31,7 +32,7 @@ def test_matches_oracle(torch_cuda, oracle, prec, nb, nmax):  # noqa: F811
     assert rel_err(got, ref, unc, empty_slabs(pos, edges)).max() < TOL[prec]
 
 
-@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "f16x3"])
 def test_alternating_output_slots(torch_cuda, prec):  # noqa: F811
     """Catalogues that alternate between two output slots add up in each slot as they do alone."""
     from paper_2509_07974_gb300 import ext4pcf
