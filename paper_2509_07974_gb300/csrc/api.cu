@@ -881,11 +881,11 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
         Q.seg[q].cell_start = G.cells + G.coff[Q.seg[q].cat];
       }
       if (f64) {
-        GK(gather_wave<double>(G.cat, cat, G.bins, L, Q, pi > 0, (double2*)ctx->rec.p, (double2*)ctx->xw.p,
-                               (unsigned long long*)ctx->counter.p, ctx->sm_count, s));
+        GK(gather_wave64(G.cat, cat, G.bins, L, Q, pi > 0, (double2*)ctx->rec.p, (double2*)ctx->xw.p,
+                               (unsigned long long*)ctx->counter.p, s));
       } else {
-        GK(gather_wave<float>(G.cat, cat, G.bins, L, Q, pi > 0, (float2*)ctx->rec.p, (float2*)ctx->xw.p,
-                              (unsigned long long*)ctx->counter.p, ctx->sm_count, s));
+        GK(gather_wave32(G.cat, cat, G.bins, L, Q, pi > 0, (float2*)ctx->rec.p, (float2*)ctx->xw.p,
+                              (unsigned long long*)ctx->counter.p, s));
       }
     }
     if (records) {  // the wave's records to the output, at the centres' places in the request
@@ -1192,13 +1192,13 @@ int ext4pcf_measure3(ext4pcf_ctx* ctx, const double* positions, const double* sh
     P.seg[0] = WaveSeg{(const int*)ctx->centres.p, nullptr, (const GridGeom*)ctx->geom.p, (const int*)ctx->cell_start.p,
                        w0, Tw, 0, 0, 0};
     if (f64) {
-      GK(gather_wave<double>(cat, cat, bins, L, P, false, (double2*)ctx->rec.p, (double2*)ctx->xw.p,
-                             (unsigned long long*)ctx->counter.p, ctx->sm_count, s));
+      GK(gather_wave64(cat, cat, bins, L, P, false, (double2*)ctx->rec.p, (double2*)ctx->xw.p,
+                             (unsigned long long*)ctx->counter.p, s));
       CK(contract3_wave(L, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, Tw, upsilon3,
                         (double2*)ctx->corr.p, s));
     } else {
-      GK(gather_wave<float>(cat, cat, bins, L, P, false, (float2*)ctx->rec.p, (float2*)ctx->xw.p,
-                            (unsigned long long*)ctx->counter.p, ctx->sm_count, s));
+      GK(gather_wave32(cat, cat, bins, L, P, false, (float2*)ctx->rec.p, (float2*)ctx->xw.p,
+                            (unsigned long long*)ctx->counter.p, s));
       CK(contract3_wave(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, Tw, upsilon3,
                         (double2*)ctx->corr.p, s));
     }

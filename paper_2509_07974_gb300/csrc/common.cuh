@@ -226,15 +226,17 @@ cudaError_t reduce_batch(const double* pos, const double* shear, const double* w
                          const double* bbox, double delta, GridGeom* geoms, GridBuffers& gb, unsigned* head,
                          double* rpos, double* rshear, double* rw, int* counts, int* status, cudaStream_t s);
 
-// gather.cu: per-centre multipole records of a wave (records of padding centres are left
-// untouched).  cat: the neighbours' concatenated sorted arrays, whose grids the plan's segments
-// give; cen: the arrays the centre lists index (the same, or the galaxies when the neighbours
-// are a reduced catalogue); bins: the pass's bins (bins outside its range have zero width);
-// accumulate: add into the records instead of writing them (and the centres' x, w)
-template <typename R>
-cudaError_t gather_wave(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
-                        const WavePlan& plan, bool accumulate, cplx_t<R>* rec, cplx_t<R>* xw,
-                        unsigned long long* pair_count, int sm_count, cudaStream_t s);
+// gather.cu (FP32), gather64.cu (FP64): per-centre multipole records of a wave (records of padding
+// centres are left untouched).  cat: the neighbours' concatenated sorted arrays, whose grids the
+// plan's segments give; cen: the arrays the centre lists index (the same, or the galaxies when the
+// neighbours are a reduced catalogue); bins: the pass's bins (bins outside its range have zero
+// width); accumulate: add into the records instead of writing them (and the centres' x, w)
+cudaError_t gather_wave32(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
+                          const WavePlan& plan, bool accumulate, float2* rec, float2* xw,
+                          unsigned long long* pair_count, cudaStream_t s);
+cudaError_t gather_wave64(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
+                          const WavePlan& plan, bool accumulate, double2* rec, double2* xw,
+                          unsigned long long* pair_count, cudaStream_t s);
 
 // contract.cu: a wave's independent sums (basis.cuh), added into the reduced array of its slot
 struct Basis;

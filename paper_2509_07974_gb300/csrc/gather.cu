@@ -1,4 +1,4 @@
-// Neighbour gather: for each centre galaxy i of a wave, the spin-weighted multipoles
+// FP32 neighbour gather: for each centre galaxy i of a wave, the spin-weighted multipoles
 //   G_n(theta_i, Theta) = sum_j x_j e^{i n phi_ij},   x_j = w_j gamma_c,j
 // of its neighbours in every radial bin, plus W_n and the quantities that the
 // multiple-counting corrections need (paper Eq. 4PCFUpsilon0 ff., Table tab:4PCFMCCorr).
@@ -21,11 +21,9 @@
 //   (c) the triple terms, split over the power blocks in FP32, are summed in block order,
 //       and the record is written to the wave buffer (or added to it, for the later passes
 //       of the tree approximation).
-// FP64 variant: positions and arithmetic in double; the bin decision r^2 = dx*dx + dy*dy is
-// evaluated with two rounded products and one rounded sum, as the FP64 definition reads.
-// FP32 variant: positions are cell-anchored floats (cell offset exact, in-cell offset
-// rounded), so dx is accurate to ~1e-7 of the cell size; pairs whose r^2 lies within a few
-// rounding errors of a bin edge are re-decided from the double positions.
+// Positions are cell-anchored floats (cell offset exact, in-cell offset rounded), so dx is accurate
+// to ~1e-7 of the cell size; pairs whose r^2 lies within a few rounding errors of a bin edge are
+// re-decided from the double positions.  (gather64.cu: the FP64 form.)
 #include "common.cuh"
 #include "gather_common.cuh"
 
@@ -34,150 +32,47 @@ namespace ext4pcf {
 namespace {
 
 constexpr int kThreads = 256;
-// FP32 (6-power blocks) splits the triple terms over the power blocks: partial sums per
-// (bin, block) in shared memory, added in block order at the end of the centre
-template <typename R, int MB> constexpr bool kTrSplitOf = sizeof(R) == 4 && MB >= 6;
+constexpr int kMB = 6;  // powers per block
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
 // Bucketed pairs in shared memory, structure of arrays: uv = (u_re, u_im, v_re, v_im) with
 // u = e^{i phi}, v = u^mb; x = w gamma_c; w.  28 bytes per pair in FP32.
-template <typename R> struct Vec4;
-template <> struct Vec4<float> { using T = float4; };
-struct __align__(16) Dbl4 { double x, y, z, w; };
-template <> struct Vec4<double> { using T = Dbl4; };
-template <typename R> struct EntArrays {
-  typename Vec4<R>::T* uv;
-  cplx_t<R>* x;
-  R* w;
-};
 
-template <typename R, int MB> struct GCfg {
-  static constexpr int kRaw = 14 * MB + 10;
-  static constexpr int V = (kRaw + 31) / 32 * 32;
-};
-
-template <typename R>
-__device__ __forceinline__ void cpow(R br, R bi, int e, R& pr, R& pi) {
-  pr = R(1); pi = R(0);
-  while (e) {
-    if (e & 1) { R t = pr * br - pi * bi; pi = pr * bi + pi * br; pr = t; }
-    R t = br * br - bi * bi; bi = R(2) * br * bi; br = t;
-    e >>= 1;
-  }
-}
+// sums of an item (14 per power, 10 triple terms), rounded up to whole lanes
+constexpr int V = (14 * kMB + 10 + 31) / 32 * 32;
 
 // u^e for 0 <= e < 32 by binary powering, unrolled (e is uniform across the warp)
-template <typename R>
-__device__ __forceinline__ void cpow5(R br, R bi, int e, R& pr, R& pi) {
-  pr = R(1); pi = R(0);
+__device__ __forceinline__ void cpow5(float br, float bi, int e, float& pr, float& pi) {
+  pr = 1.f; pi = 0.f;
 #pragma unroll
   for (int bit = 0; bit < 5; ++bit) {
-    if (e & (1 << bit)) { R t = pr * br - pi * bi; pi = pr * bi + pi * br; pr = t; }
-    if (e >> (bit + 1)) { R t = br * br - bi * bi; bi = R(2) * br * bi; br = t; }
+    if (e & (1 << bit)) { float t = pr * br - pi * bi; pi = pr * bi + pi * br; pr = t; }
+    if (e >> (bit + 1)) { float t = br * br - bi * bi; bi = 2.f * br * bi; br = t; }
   }
 }
 
 // transposed butterfly: after the call lane l holds in a[0..V/32) the warp totals of the
 // original slots j + base(l), base(l) = sum_k bit_k(l) * V / 2^(5-k)
-template <typename R, int V, int OFF>
-__device__ __forceinline__ void rt_step(R* a, int lane) {
-  constexpr int H = V / 2;
+template <int W, int OFF>
+__device__ __forceinline__ void rt_step(float* a, int lane) {
+  constexpr int H = W / 2;
   const bool up = (lane & OFF) != 0;
 #pragma unroll
   for (int j = 0; j < H; ++j) {
-    R send = up ? a[j] : a[j + H];
-    R keep = up ? a[j + H] : a[j];
+    const float send = up ? a[j] : a[j + H];
+    const float keep = up ? a[j + H] : a[j];
     a[j] = keep + __shfl_xor_sync(kFull, send, OFF);
   }
 }
-template <typename R, int V>
-__device__ __forceinline__ void reduce_transpose(R* a, int lane) {
-  rt_step<R, V, 16>(a, lane);
-  rt_step<R, V / 2, 8>(a, lane);
-  rt_step<R, V / 4, 4>(a, lane);
-  rt_step<R, V / 8, 2>(a, lane);
-  rt_step<R, V / 16, 1>(a, lane);
+__device__ __forceinline__ void reduce_transpose(float* a, int lane) {
+  rt_step<V, 16>(a, lane);
+  rt_step<V / 2, 8>(a, lane);
+  rt_step<V / 4, 4>(a, lane);
+  rt_step<V / 8, 2>(a, lane);
+  rt_step<V / 16, 1>(a, lane);
 }
 
-
-// FP32 pass-3 inner loop with packed pairs: every (Re, Im) accumulator pair takes one
-// two-lane fused multiply-add per pair of the bin (each lane rounds like a scalar FFMA), and
-// the power recurrence u^{m+1} = u^m u runs on the pair (Re, Im) as one packed multiply and
-// one packed multiply-add.  Fills a[0, 14 MB + 10) in the slot order of the scalar path.
-template <int MB>
-__device__ __forceinline__ void accumulate_f32x2(float* a, const float4* __restrict__ euv,
-                                                 const float2* __restrict__ ex, const float* __restrict__ ew,
-                                                 int s0, int s1, int lane, int k, int mb, bool first) {
-  float2 acc[7 * MB];
-#pragma unroll
-  for (int j = 0; j < 7 * MB; ++j) acc[j] = make_float2(0.f, 0.f);
-  float tr[10];
-#pragma unroll
-  for (int j = 0; j < 10; ++j) tr[j] = 0.f;
-  for (int e0 = s0 + lane; e0 < s1; e0 += 64) {
-    const int e1 = e0 + 32;
-    const bool two = e1 < s1;
-    const int e1c = two ? e1 : e0;
-    const float4 q0 = euv[e0], q1 = euv[e1c];
-    const float2 xx0 = ex[e0], xx1 = ex[e1c];
-    const float w0 = ew[e0];
-    // the second pair adds nothing when it is absent
-    const float xr1 = two ? xx1.x : 0.f, xi1 = two ? xx1.y : 0.f, w1 = two ? ew[e1c] : 0.f;
-    float2 P0, P1;
-    cpow5<float>(q0.z, q0.w, k, P0.x, P0.y);
-    cpow5<float>(q1.z, q1.w, k, P1.x, P1.y);
-    const float2 U0 = make_float2(q0.x, q0.y), U0s = make_float2(-q0.y, q0.x);
-    const float2 U1 = make_float2(q1.x, q1.y), U1s = make_float2(-q1.y, q1.x);
-    const float wt0[7] = {xx0.x, xx0.y, xx0.x * xx0.x - xx0.y * xx0.y, 2.f * xx0.x * xx0.y, w0,
-                          xx0.x * xx0.x + xx0.y * xx0.y, w0 * w0};
-    const float wt1[7] = {xr1, xi1, xr1 * xr1 - xi1 * xi1, 2.f * xr1 * xi1, w1, xr1 * xr1 + xi1 * xi1, w1 * w1};
-    auto step = [&](int t) {
-#pragma unroll
-      for (int q = 0; q < 7; ++q) {
-        acc[7 * t + q] = __ffma2_rn(make_float2(wt0[q], wt0[q]), P0, acc[7 * t + q]);
-        acc[7 * t + q] = __ffma2_rn(make_float2(wt1[q], wt1[q]), P1, acc[7 * t + q]);
-      }
-      P0 = __ffma2_rn(make_float2(P0.x, P0.x), U0, __fmul2_rn(make_float2(P0.y, P0.y), U0s));
-      P1 = __ffma2_rn(make_float2(P1.x, P1.x), U1, __fmul2_rn(make_float2(P1.y, P1.y), U1s));
-    };
-    if (mb == MB) {
-#pragma unroll
-      for (int t = 0; t < MB; ++t) step(t);
-    } else {
-#pragma unroll
-      for (int t = 0; t < MB; ++t)
-        if (t < mb) step(t);
-    }
-    if (first) {
-      // x^3 u^-8, x^3 u^-4, x^2 x^* u^-4, x^2 x^*, w^3 (the second pair is zero if absent)
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float ur = q ? q1.x : q0.x, ui = q ? q1.y : q0.y;
-        const float* wt = q ? wt1 : wt0;
-        const float xr = wt[0], xi = wt[1], x2r = wt[2], x2i = wt[3], ww = wt[4], xa = wt[5], w2 = wt[6];
-        float u2r = ur * ur - ui * ui, u2i = 2.f * ur * ui;
-        float u4r = u2r * u2r - u2i * u2i, u4i = 2.f * u2r * u2i;
-        float u8r = u4r * u4r - u4i * u4i, u8i = 2.f * u4r * u4i;
-        float x3r = x2r * xr - x2i * xi, x3i = x2r * xi + x2i * xr;
-        float xcr = xa * xr, xci = xa * xi;  // x^2 x^* = |x|^2 x
-        tr[0] += x3r * u8r + x3i * u8i;  // x3 * conj(u8)
-        tr[1] += x3i * u8r - x3r * u8i;
-        tr[2] += x3r * u4r + x3i * u4i;
-        tr[3] += x3i * u4r - x3r * u4i;
-        tr[4] += xcr * u4r + xci * u4i;
-        tr[5] += xci * u4r - xcr * u4i;
-        tr[6] += xcr;
-        tr[7] += xci;
-        tr[8] += w2 * ww;
-      }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 7 * MB; ++j) { a[2 * j] = acc[j].x; a[2 * j + 1] = acc[j].y; }
-#pragma unroll
-  for (int j = 0; j < 10; ++j) a[14 * MB + j] = tr[j];
-}
 
 // v^k for the block index k (uniform across the warp): the shortest product chain for
 // k < 8 as straight-line code behind one uniform branch, binary powering beyond
@@ -195,17 +90,18 @@ __device__ __forceinline__ void vpow_block(float vr, float vi, int k, float2& P)
     case 5: { const float2 v2 = cmul_f(v, v); P = cmul_f(cmul_f(v2, v2), v); return; }
     case 6: { const float2 v2 = cmul_f(v, v); P = cmul_f(cmul_f(v2, v2), v2); return; }
     case 7: { const float2 v2 = cmul_f(v, v); P = cmul_f(cmul_f(cmul_f(v2, v2), v2), v); return; }
-    default: cpow5<float>(vr, vi, k, P.x, P.y); return;
+    default: cpow5(vr, vi, k, P.x, P.y); return;
   }
 }
 
-// FP32 pass-3 inner loop, one pair per lane per iteration (for larger power blocks: the
-// per-pair set-up -- loads, the block's first power, the weights -- is paid once per block
-// of MB powers).  Fills a[0, 14 MB + 10) in the slot order of the scalar path.
-template <int MB>
-__device__ __forceinline__ void accumulate1_f32x2(float* a, const float4* __restrict__ euv,
-                                                  const float2* __restrict__ ex, const float* __restrict__ ew,
-                                                  int s0, int s1, int lane, int k, int mb, int tr_nsub) {
+// The sums of one item, one pair per lane and iteration, with packed pairs: every (Re, Im)
+// accumulator pair takes one two-lane fused multiply-add per pair of the bin (each lane rounds like
+// a scalar FFMA), and the power recurrence u^{m+1} = u^m u runs on the pair (Re, Im) as one packed
+// multiply and one packed multiply-add.  Fills a[0, 14 kMB) power by power, then the triple terms.
+__device__ __forceinline__ void accumulate(float* a, const float4* __restrict__ euv, const float2* __restrict__ ex,
+                                           const float* __restrict__ ew, int s0, int s1, int lane, int k, int mb,
+                                           int tr_nsub) {
+  constexpr int MB = kMB;
   float2 acc[7 * MB];
 #pragma unroll
   for (int j = 0; j < 7 * MB; ++j) acc[j] = make_float2(0.f, 0.f);
@@ -268,21 +164,19 @@ __device__ __forceinline__ void accumulate1_f32x2(float* a, const float4* __rest
   for (int j = 0; j < 10; ++j) a[14 * MB + j] = tr[j];
 }
 
-template <typename R, int MB, int MINB>
-__global__ void __launch_bounds__(kThreads, MINB)
-gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __restrict__ xw) {
-  using Cx = cplx_t<R>;
-  constexpr int V = GCfg<R, MB>::V;
+// two CTAs of 8 warps per SM: 6 powers per block keep the accumulators within 128 registers, and
+// each CTA gets half of the shared memory
+__global__ void __launch_bounds__(kThreads, 2)
+gather_kernel(const GatherArgs args, float2* __restrict__ rec, float2* __restrict__ xw) {
   extern __shared__ __align__(16) unsigned char smem[];
   const SortedCat& cat = args.cat;
   const Layout L = args.L;
   const int nb = args.bins.nb, cap = args.cap, mb = args.mb, nblk = args.nblk;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  using V4 = typename Vec4<R>::T;
-  V4* euv = reinterpret_cast<V4*>(smem);
-  Cx* ex = reinterpret_cast<Cx*>(euv + cap);
-  R* ew = reinterpret_cast<R*>(ex + cap);
+  float4* euv = reinterpret_cast<float4*>(smem);
+  float2* ex = reinterpret_cast<float2*>(euv + cap);
+  float* ew = reinterpret_cast<float*>(ex + cap);
   double* e2 = reinterpret_cast<double*>(ew + cap);
   float* e2f = reinterpret_cast<float*>(e2 + 65);
   float* win = e2f + 65;
@@ -293,11 +187,10 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
   int* misc = rpre + kMaxRows + 1;  // rows, candidates, work items taken
   int* fidx = misc + 8;             // [nblk][V] where the reduced slots of each power block go
   // partial sums of the split triple terms: trs [nb][nblk][10]
-  constexpr bool kTrSplit = kTrSplitOf<R, MB>;
-  R* trs = reinterpret_cast<R*>(fidx + nblk * V);
-  unsigned char* btab = reinterpret_cast<unsigned char*>(trs + (kTrSplit ? nb * nblk * 10 : 0));  // [256]
+  float* trs = reinterpret_cast<float*>(fidx + nblk * V);
+  unsigned char* btab = reinterpret_cast<unsigned char*>(trs + nb * nblk * 10);  // [256]
   signed char* cbin = reinterpret_cast<signed char*>(btab + 256);  // bin of each candidate
-  Cx* accs = reinterpret_cast<Cx*>((reinterpret_cast<uintptr_t>(cbin + cap) + 15) & ~(uintptr_t)15);
+  float2* accs = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(cbin + cap) + 15) & ~(uintptr_t)15);
 
   for (int b = tid; b <= nb; b += kThreads) {
     e2[b] = args.bins.e2[b]; e2f[b] = args.bins.e2f[b];
@@ -322,7 +215,7 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
   for (int i = tid; i < nblk * V; i += kThreads) {
     const int k = i / V, slot = i % V, m0 = k * mb;
     int f = -1;
-    if (slot < 14 * MB) {
+    if (slot < 14 * kMB) {
       const int t = slot / 14, q = slot % 14, m = m0 + t;
       int idx = -1;
       if (t < mb) {
@@ -330,16 +223,15 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
           case 0: if (m <= 2 * L.N - 1) idx = L.G(m, 0); break;
           case 1: if (m >= 1 && m <= 2 * L.N + 3) idx = L.G(-m, 0); break;
           case 2: if (m <= 2 * L.N - 2) idx = L.XX(m, 0); break;
-          case 3: if (m >= 1 && m <= 2 * L.N + 6) idx = L.XX(-m, 0); break;
+          case 3: if (m >= 1 && -m <= 2 * L.N - 2 && m <= 2 * L.N + 6) idx = L.XX(-m, 0); break;
           case 4: if (m <= 2 * L.N) idx = L.W(m, 0); break;
           case 5: if (m <= 2 * L.N + 2) idx = L.XA(m, 0); break;
           default: if (m <= 2 * L.N) idx = L.WW(m, 0); break;
         }
       }
       f = idx >= 0 ? 2 * idx + (slot & 1) : -1;
-    } else if (slot < 14 * MB + 10) {
-      if (kTrSplit) f = -2 - (slot - 14 * MB);
-      else f = m0 == 0 ? 2 * L.TR((slot - 14 * MB) >> 1, 0) + (slot & 1) : -1;
+    } else if (slot < 14 * kMB + 10) {
+      f = -2 - (slot - 14 * kMB);
     }
     fidx[i] = f;
   }
@@ -372,13 +264,10 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
     const double pxi = args.cen.px[pi], pyi = args.cen.py[pi];
     // the centre in the neighbours' grid frame: cell corner and offset as float, by the
     // arithmetic that builds the neighbours' (cell corner, offset) pairs
-    float4 Pi = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (sizeof(R) == 4) {
-      const int ccx = min(max((int)floor((pxi - gx0) * gm.inv_cell), 0), gncx - 1);
-      const int ccy = min(max((int)floor((pyi - gy0) * gm.inv_cell), 0), gncy - 1);
-      Pi = make_float4((float)ccx * gm.cellf, (float)ccy * gm.cellf, (float)((pxi - gx0) - (double)ccx * cell),
-                       (float)((pyi - gy0) - (double)ccy * cell));
-    }
+    const int ccx = min(max((int)floor((pxi - gx0) * gm.inv_cell), 0), gncx - 1);
+    const int ccy = min(max((int)floor((pyi - gy0) * gm.inv_cell), 0), gncy - 1);
+    const float4 Pi = make_float4((float)ccx * gm.cellf, (float)ccy * gm.cellf,
+                                  (float)((pxi - gx0) - (double)ccx * cell), (float)((pyi - gy0) - (double)ccy * cell));
     if (warp == 0) {
       // the rows of cells within rmax of the centre, one per lane (cells are at least rmax / 16
       // wide, so there are at most 34), kept in row order when they hold galaxies
@@ -424,11 +313,10 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
       }
     }
     // the record collects in shared memory
-    Cx* dst = rec + (size_t)c * L.rec;
-    R* accf = reinterpret_cast<R*>(accs);
-    for (int k = tid; k < L.rec; k += kThreads) accs[k] = cmk<Cx>(R(0), R(0));
-    if (kTrSplit)
-      for (int i = tid; i < nb * nblk * 10; i += kThreads) trs[i] = R(0);
+    float2* dst = rec + (size_t)c * L.rec;
+    float* accf = reinterpret_cast<float*>(accs);
+    for (int k = tid; k < L.rec; k += kThreads) accs[k] = make_float2(0.f, 0.f);
+    for (int i = tid; i < nb * nblk * 10; i += kThreads) trs[i] = 0.f;
     __syncthreads();
     const int nr = misc[0], total = misc[1];
     unsigned long long pairs_here = 0;
@@ -437,17 +325,15 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
       // ---- classification and stable bucketing by bin of the next cap candidates
       const int cend = min(total, cpos + cap);
       if (tid == 0) misc[2] = 0;  // work items of this chunk taken so far (read after the barriers below)
-      bucket_chunk<R, kWarps>(cat, rstart, rpre, nr, cpos, cend, pxi, pyi, Pi, e2, e2f, win, lk, nb, cbin, wcnt, off,
-                              [&](int dst, R ur, R ui, int q) {
-                                R xr, xi, ww, vr, vi;
-                                Pair<R>::load_x(cat, q, xr, xi, ww);
-                                cpow5<R>(ur, ui, mb, vr, vi);
-                                V4 e;
-                                e.x = ur; e.y = ui; e.z = vr; e.w = vi;
-                                euv[dst] = e;
-                                ex[dst] = cmk<Cx>(xr, xi);
-                                ew[dst] = ww;
-                              });
+      bucket_chunk<float, kWarps>(cat, rstart, rpre, nr, cpos, cend, pxi, pyi, Pi, e2, e2f, win, lk, nb, cbin, wcnt,
+                                  off, [&](int dst, float ur, float ui, int q) {
+                                    float xr, xi, ww, vr, vi;
+                                    Pair<float>::load_x(cat, q, xr, xi, ww);
+                                    cpow5(ur, ui, mb, vr, vi);
+                                    euv[dst] = make_float4(ur, ui, vr, vi);
+                                    ex[dst] = make_float2(xr, xi);
+                                    ew[dst] = ww;
+                                  });
       // ---- pass 3: the work items (bin, power block) of the chunk, outer bins (the fuller
       // ones) first, each taken by the next free warp; an item's sums go straight into the
       // record, whose entries no other item of the chunk touches
@@ -459,123 +345,39 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
         // the warp's next item is requested now and used at the end of this one
         int next = 0;
         if (lane == 0) next = atomicAdd(&misc[2], 1);
-        const int b = nb - 1 - item / nblk, k = item % nblk, m0 = k * mb;
+        const int b = nb - 1 - item / nblk, k = item % nblk;
         const int s0 = off[b], s1 = off[b + 1];
         if (s0 < s1) {
-          R a[V];
+          float a[V];
 #pragma unroll
-          for (int j = 0; j < V; ++j) a[j] = R(0);
-          // two pairs per lane and iteration: two independent power recurrences
-          auto accumulate = [&](int e0, int e1) {
-            if constexpr (sizeof(R) == 4) return;  // the FP32 path runs accumulate_f32x2
-            const bool two = e1 < s1;
-            const int e1c = two ? e1 : e0;
-            const V4 q0 = euv[e0], q1 = euv[e1c];
-            const Cx xx0 = ex[e0], xx1 = ex[e1c];
-            const R ur0 = q0.x, ui0 = q0.y, vr0 = q0.z, vi0 = q0.w;
-            const R ur1 = q1.x, ui1 = q1.y, vr1 = q1.z, vi1 = q1.w;
-            const R xr0 = xx0.x, xi0 = xx0.y, w0 = ew[e0];
-            // the second pair adds nothing when it is absent
-            const R xr1 = two ? xx1.x : R(0), xi1 = two ? xx1.y : R(0), w1 = two ? ew[e1c] : R(0);
-            R pr0, pi0, pr1, pi1;
-            cpow5<R>(vr0, vi0, k, pr0, pi0);
-            cpow5<R>(vr1, vi1, k, pr1, pi1);
-            const R x2r0 = xr0 * xr0 - xi0 * xi0, x2i0 = R(2) * xr0 * xi0, xa0 = xr0 * xr0 + xi0 * xi0;
-            const R x2r1 = xr1 * xr1 - xi1 * xi1, x2i1 = R(2) * xr1 * xi1, xa1 = xr1 * xr1 + xi1 * xi1;
-            const R ww0 = w0 * w0, ww1 = w1 * w1;
-            // one power at a time; every slot is updated by two separate multiply-adds
-            // (a sum of products would cost a multiply, a fused multiply-add and an add)
-            auto step = [&](int t) {
-              a[14 * t + 0] += xr0 * pr0;   a[14 * t + 0] += xr1 * pr1;
-              a[14 * t + 1] += xr0 * pi0;   a[14 * t + 1] += xr1 * pi1;
-              a[14 * t + 2] += xi0 * pr0;   a[14 * t + 2] += xi1 * pr1;
-              a[14 * t + 3] += xi0 * pi0;   a[14 * t + 3] += xi1 * pi1;
-              a[14 * t + 4] += x2r0 * pr0;  a[14 * t + 4] += x2r1 * pr1;
-              a[14 * t + 5] += x2r0 * pi0;  a[14 * t + 5] += x2r1 * pi1;
-              a[14 * t + 6] += x2i0 * pr0;  a[14 * t + 6] += x2i1 * pr1;
-              a[14 * t + 7] += x2i0 * pi0;  a[14 * t + 7] += x2i1 * pi1;
-              a[14 * t + 8] += w0 * pr0;    a[14 * t + 8] += w1 * pr1;
-              a[14 * t + 9] += w0 * pi0;    a[14 * t + 9] += w1 * pi1;
-              a[14 * t + 10] += xa0 * pr0;  a[14 * t + 10] += xa1 * pr1;
-              a[14 * t + 11] += xa0 * pi0;  a[14 * t + 11] += xa1 * pi1;
-              a[14 * t + 12] += ww0 * pr0;  a[14 * t + 12] += ww1 * pr1;
-              a[14 * t + 13] += ww0 * pi0;  a[14 * t + 13] += ww1 * pi1;
-              const R n0 = pr0 * ur0 - pi0 * ui0;
-              pi0 = pr0 * ui0 + pi0 * ur0;
-              pr0 = n0;
-              const R n1 = pr1 * ur1 - pi1 * ui1;
-              pi1 = pr1 * ui1 + pi1 * ur1;
-              pr1 = n1;
-            };
-            if (mb == MB) {  // the common case: a full block, no predicates
-#pragma unroll
-              for (int t = 0; t < MB; ++t) step(t);
-            } else {
-#pragma unroll
-              for (int t = 0; t < MB; ++t)
-                if (t < mb) step(t);
-            }
-            if (m0 == 0) {
-              // x^3 u^-8, x^3 u^-4, x^2 x^* u^-4, x^2 x^*, w^3 (the second pair is zero if absent)
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                const R ur = q ? ur1 : ur0, ui = q ? ui1 : ui0, xr = q ? xr1 : xr0, xi = q ? xi1 : xi0;
-                const R x2r = q ? x2r1 : x2r0, x2i = q ? x2i1 : x2i0, xa = q ? xa1 : xa0;
-                const R ww = q ? w1 : w0, w2 = q ? ww1 : ww0;
-                R u2r = ur * ur - ui * ui, u2i = R(2) * ur * ui;
-                R u4r = u2r * u2r - u2i * u2i, u4i = R(2) * u2r * u2i;
-                R u8r = u4r * u4r - u4i * u4i, u8i = R(2) * u4r * u4i;
-                R x3r = x2r * xr - x2i * xi, x3i = x2r * xi + x2i * xr;
-                R xcr = xa * xr, xci = xa * xi;  // x^2 x^* = |x|^2 x
-                constexpr int o = 14 * MB;
-                a[o + 0] += x3r * u8r + x3i * u8i;  // x3 * conj(u8)
-                a[o + 1] += x3i * u8r - x3r * u8i;
-                a[o + 2] += x3r * u4r + x3i * u4i;
-                a[o + 3] += x3i * u4r - x3r * u4i;
-                a[o + 4] += xcr * u4r + xci * u4i;
-                a[o + 5] += xci * u4r - xcr * u4i;
-                a[o + 6] += xcr;
-                a[o + 7] += xci;
-                a[o + 8] += w2 * ww;
-              }
-            }
-          };
-          if constexpr (kTrSplit)
-            accumulate1_f32x2<MB>(reinterpret_cast<float*>(a), reinterpret_cast<const float4*>(euv),
-                                  reinterpret_cast<const float2*>(ex), reinterpret_cast<const float*>(ew), s0,
-                                  s1, lane, k, mb, args.nblk);
-          else if constexpr (sizeof(R) == 4)
-            accumulate_f32x2<MB>(reinterpret_cast<float*>(a), reinterpret_cast<const float4*>(euv),
-                                 reinterpret_cast<const float2*>(ex), reinterpret_cast<const float*>(ew), s0,
-                                 s1, lane, k, mb, m0 == 0);
-          else
-            for (int e = s0 + lane; e < s1; e += 64) accumulate(e, e + 32);
+          for (int j = 0; j < V; ++j) a[j] = 0.f;
+          accumulate(a, euv, ex, ew, s0, s1, lane, k, mb, nblk);
           // the item's record entries (their current values load while the lanes reduce)
           int f[V / 32];
-          R cur[V / 32];
+          float cur[V / 32];
 #pragma unroll
           for (int j = 0; j < V / 32; ++j) {
             f[j] = fidx[k * V + rbase + j];
-            cur[j] = f[j] >= 0 ? accf[f[j] + 2 * b] : R(0);
+            cur[j] = f[j] >= 0 ? accf[f[j] + 2 * b] : 0.f;
           }
           // with R = sum Re(x) u^m = (a0, a1) and I = sum Im(x) u^m = (a2, a3):
           //   sum x u^m = (a0 - a3, a1 + a2),  sum x conj(u^m) = (a0 + a3, a2 - a1)
 #pragma unroll
-          for (int t = 0; t < MB; ++t) {
+          for (int t = 0; t < kMB; ++t) {
 #pragma unroll
             for (int q = 0; q < 8; q += 4) {
-              const R r0 = a[14 * t + q], r1 = a[14 * t + q + 1], i0 = a[14 * t + q + 2], i1 = a[14 * t + q + 3];
+              const float r0 = a[14 * t + q], r1 = a[14 * t + q + 1], i0 = a[14 * t + q + 2], i1 = a[14 * t + q + 3];
               a[14 * t + q] = r0 - i1;
               a[14 * t + q + 1] = r1 + i0;
               a[14 * t + q + 2] = r0 + i1;
               a[14 * t + q + 3] = i0 - r1;
             }
           }
-          reduce_transpose<R, V>(a, lane);
+          reduce_transpose(a, lane);
 #pragma unroll
           for (int j = 0; j < V / 32; ++j) {
             if (f[j] >= 0) accf[f[j] + 2 * b] = cur[j] + a[j];
-            else if (kTrSplit && f[j] <= -2) trs[(b * nblk + k) * 10 + (-2 - f[j])] += a[j];
+            else if (f[j] <= -2) trs[(b * nblk + k) * 10 + (-2 - f[j])] += a[j];
           }
         }
         item = __shfl_sync(kFull, next, 0);
@@ -584,14 +386,12 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
       cpos = cend;
       __syncthreads();
     }
-    if (kTrSplit) {
-      // triple terms: the power blocks' sums, in block order
-      for (int i = tid; i < nb * 10; i += kThreads) {
-        const int b = i / 10, q = i % 10;
-        R sum = R(0);
-        for (int k = 0; k < nblk; ++k) sum += trs[(b * nblk + k) * 10 + q];
-        accf[2 * L.TR(q >> 1, b) + (q & 1)] += sum;
-      }
+    // triple terms: the power blocks' sums, in block order
+    for (int i = tid; i < nb * 10; i += kThreads) {
+      const int b = i / 10, q = i % 10;
+      float sum = 0.f;
+      for (int k = 0; k < nblk; ++k) sum += trs[(b * nblk + k) * 10 + q];
+      accf[2 * L.TR(q >> 1, b) + (q & 1)] += sum;
     }
     __syncthreads();
     if (args.accumulate) {
@@ -600,10 +400,10 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
       for (int k = tid; k < L.rec; k += kThreads) dst[k] = accs[k];
     }
     if (tid == 0 && !args.accumulate) {
-      R xr, xi, ww;
-      Pair<R>::load_x(args.cen, pi, xr, xi, ww);
-      xw[2 * (size_t)c] = cmk<Cx>(xr, xi);
-      xw[2 * (size_t)c + 1] = cmk<Cx>(ww, R(0));
+      float xr, xi, ww;
+      Pair<float>::load_x(args.cen, pi, xr, xi, ww);
+      xw[2 * (size_t)c] = make_float2(xr, xi);
+      xw[2 * (size_t)c + 1] = make_float2(ww, 0.f);
     }
     if (tid == 0) {
       atomicAdd(args.pair_count, pairs_here);
@@ -612,54 +412,34 @@ gather_kernel(const GatherArgs args, cplx_t<R>* __restrict__ rec, cplx_t<R>* __r
   }
 }
 
-// powers per warp block and resident CTAs per SM: FP32 runs two CTAs of 8 warps per SM
-// (3 powers per block keep the accumulators within 128 registers, and each CTA gets half
-// of the shared memory), FP64 one CTA with 3 powers per block
-template <typename R> constexpr int kMB = sizeof(R) == 4 ? 6 : 3;
-template <typename R> constexpr int kMinBlocks = sizeof(R) == 4 ? 2 : 1;
-
 }  // namespace
 
-template <typename R>
-cudaError_t gather_wave(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
-                        const WavePlan& plan, bool accumulate, cplx_t<R>* rec, cplx_t<R>* xw,
-                        unsigned long long* pair_count, int sm_count, cudaStream_t s) {
+cudaError_t gather_wave32(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
+                          const WavePlan& plan, bool accumulate, float2* rec, float2* xw,
+                          unsigned long long* pair_count, cudaStream_t s) {
   if (plan.total <= 0) return cudaSuccess;
-  constexpr int MB = kMB<R>;
-  constexpr int MINB = kMinBlocks<R>;
   GatherArgs a;
   a.cat = cat; a.cen = cen; a.accumulate = accumulate ? 1 : 0;
   a.bins = bins; a.L = L; a.plan = plan; a.pair_count = pair_count;
   const int npow = L.max_pow + 1;
-  const int nblk = (npow + MB - 1) / MB;  // the warps take (bin, block) items in turn
+  const int nblk = (npow + kMB - 1) / kMB;  // the warps take (bin, block) items in turn
   a.mb = (npow + nblk - 1) / nblk;
   a.nblk = (npow + a.mb - 1) / a.mb;
-  const size_t fixed = (size_t)L.rec * sizeof(cplx_t<R>) + 16 + 65 * sizeof(double) + 130 * sizeof(float) +
-                       (65 + kWarps * 64 + 2 * kMaxRows + 1 + 8 + (size_t)a.nblk * GCfg<R, MB>::V) * sizeof(int) + 256 +
-                       64 + (kTrSplitOf<R, MB> ? (size_t)bins.nb * a.nblk * 10 * sizeof(R) : 0);
-  const size_t budget = MINB == 1 ? 227 * 1024 : 113 * 1024;
-  constexpr size_t per_pair = sizeof(typename Vec4<R>::T) + sizeof(cplx_t<R>) + sizeof(R) + 1;
+  const size_t fixed = (size_t)L.rec * sizeof(float2) + 16 + 65 * sizeof(double) + 130 * sizeof(float) +
+                       (65 + kWarps * 64 + 2 * kMaxRows + 1 + 8 + (size_t)a.nblk * V) * sizeof(int) + 256 +
+                       64 + (size_t)bins.nb * a.nblk * 10 * sizeof(float);
+  const size_t budget = 113 * 1024;
+  constexpr size_t per_pair = sizeof(float4) + sizeof(float2) + sizeof(float) + 1;
   if (fixed + per_pair * kThreads > budget) return cudaErrorInvalidConfiguration;
-  int cap = (int)((budget - fixed) / per_pair);
-  cap = cap / kThreads * kThreads;
+  int cap = (int)((budget - fixed) / per_pair) / kThreads * kThreads;
   if (cap > 8192) cap = 8192;
   a.cap = cap;
   const size_t smem = fixed + (size_t)cap * per_pair;
-  cudaError_t e = cudaFuncSetAttribute(gather_kernel<R, MB, MINB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int grid = plan.total;
-  gather_kernel<R, MB, MINB><<<grid, kThreads, smem, s>>>(a, rec, xw);
+  gather_kernel<<<plan.total, kThreads, smem, s>>>(a, rec, xw);
   ++g_launches;
-  (void)sm_count;
   return cudaGetLastError();
 }
-
-template cudaError_t gather_wave<float>(const SortedCat&, const SortedCat&, const Bins&, const Layout&,
-                                        const WavePlan&, bool, float2*, float2*, unsigned long long*, int,
-                                        cudaStream_t);
-template cudaError_t gather_wave<double>(const SortedCat&, const SortedCat&, const Bins&, const Layout&,
-                                         const WavePlan&, bool, double2*, double2*, unsigned long long*, int,
-                                         cudaStream_t);
 
 }  // namespace ext4pcf

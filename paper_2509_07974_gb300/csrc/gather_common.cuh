@@ -161,8 +161,10 @@ __device__ __forceinline__ void bucket_chunk(const SortedCat& cat, const int* rs
   }
   if (lane < nb) wcnt[warp * 64 + lane] = 0;
   __syncwarp();
-  lk.out_lo = e2f[0] - win[0];
-  lk.out_hi = e2f[nb] + win[nb];
+  if (sizeof(R) == 4) {
+    lk.out_lo = e2f[0] - win[0];
+    lk.out_hi = e2f[nb] + win[nb];
+  }
   // ---- pass 1: bin of every candidate, counts per (warp, bin)
   int r = r0;
   for (int t0 = w0; t0 < w1; t0 += 32) {
