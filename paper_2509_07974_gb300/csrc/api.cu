@@ -440,7 +440,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   // time, the split-FP16 form those of every slot
   const bool cc = !tc && !records;
   const bool h16 = prec == EXT4PCF_SPLIT_F16;
-  if ((cc || h16) && (ctx->basis.N != n_max || ctx->basis.nb != n_bins || ctx->basis.npairs == 0)) {
+  if (!records && (ctx->basis.N != n_max || ctx->basis.nb != n_bins || ctx->basis.npairs == 0)) {
     if (!basis_make(L, ctx->basis)) return fail(ctx, EXT4PCF_E_UNSUPPORTED, "no reduced rows for this n_max");
   }
   if (tc) {
@@ -805,7 +805,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   }
   ENSURE(ctx->xw, (size_t)Tmax * 2 * cbytes);
   std::vector<float> trial_ms;
-  const size_t corr_doubles = corrections_size(L);
+  const size_t corr_doubles = corrections_slot_doubles(L, n_out);
   ENSURE(ctx->corr, corr_doubles * 8 * n_out);
   CK(cudaMemsetAsync(ctx->corr.p, 0, corr_doubles * 8 * n_out, s));
   const size_t red_doubles = h16 ? 2 * ctx->basis.elems() : tc ? tc_reduced_doubles(L) : 0;
@@ -864,8 +864,18 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   size_t wave_i = 0;
   WavePlan P;
   double* red_base = (double*)ctx->tc_red.p;
-  int red_slot = -1;  // output slot of the CUDA-core forms' reduced array
   double* corr_base = (double*)ctx->corr.p;
+  int red_slot = -1;  // output slot of the CUDA-core forms' reduced array
+  // its sums and their multiple-counting terms to its output, and the arrays cleared for the next
+  auto flush_slot = [&]() -> cudaError_t {
+    double* corr = corr_base + corr_doubles * (size_t)red_slot;
+    cudaError_t e = corrections_finish(L, n_out, red_slot, 1, corr_base, d_xi, s);
+    if (e == cudaSuccess)
+      e = basis_expand(ctx->basis, red_base, cc_slices, corr, d_ups + 2 * ups_elems * (size_t)red_slot, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(red_base, 0, cc_bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(corr, 0, corr_doubles * 8, s);
+    return e;
+  };
   for (;;) {
     const bool tuning = wave_i < trial.size();
     if (!next_plan(tuning ? trial[wave_i] : T, P)) break;
@@ -901,10 +911,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
     }
     if (timing) t_w1 = tmark();
     if (cc && g0.slot != red_slot) {  // the next slot: the last one's sums go to its output
-      if (red_slot >= 0) {
-        CK(basis_expand(ctx->basis, red_base, cc_slices, d_ups + 2 * ups_elems * (size_t)red_slot, s));
-        CK(cudaMemsetAsync(red_base, 0, cc_bytes, s));
-      }
+      if (red_slot >= 0) CK(flush_slot());
       red_slot = g0.slot;
     }
     if (f64) {
@@ -925,9 +932,9 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
     }
     if (timing) t_w2 = tmark();
     if (f64) {
-      CK(corrections_wave<double>(L, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, P, corr_base, d_xi, s));
+      CK(corrections_wave<double>(L, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, P, n_out, corr_base, d_xi != nullptr, s));
     } else {
-      CK(corrections_wave<float>(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, corr_base, d_xi, s));
+      CK(corrections_wave<float>(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, n_out, corr_base, d_xi != nullptr, s));
     }
     if (timing) {
       const int t_w3 = tmark();
@@ -955,13 +962,14 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   ctx->last_wave = std::min(T, largest_wave);  // the wave size in use (trial waves aside)
   if (records && rec_host && n_rec > 0)
     CK(cudaMemcpyAsync(rec_out, ctx->rec_out.p, (size_t)n_rec * L.rec * 16, cudaMemcpyDeviceToHost, s));
-  if (red_slot >= 0) CK(basis_expand(ctx->basis, red_base, cc_slices, d_ups + 2 * ups_elems * (size_t)red_slot, s));
-  // ---- per output slot: every ordered triple from the reduced array, then the corrections
-  for (int o = 0; o < n_out && !records; ++o) {
+  if (red_slot >= 0) CK(flush_slot());
+  // ---- per output slot: every ordered triple from the reduced array, less the corrections
+  if (tc && !records) CK(corrections_finish(L, n_out, 0, n_out, corr_base, d_xi, s));
+  for (int o = 0; o < n_out && tc && !records; ++o) {
     double* ups_o = d_ups + 2 * ups_elems * (size_t)o;
-    if (h16) CK(basis_expand(ctx->basis, red_base + red_doubles * (size_t)o, 1, ups_o, s));
-    else if (tc) CK(tc_expand(L, red_base + red_doubles * (size_t)o, ups_o, s));
-    CK(corrections_apply(L, corr_base + corr_doubles * (size_t)o, ups_o, s));
+    const double* corr_o = corr_base + corr_doubles * (size_t)o;
+    if (!h16) CK(tc_expand(L, red_base + red_doubles * (size_t)o, ups_o, s));
+    CK(basis_expand(ctx->basis, h16 ? red_base + red_doubles * (size_t)o : nullptr, 1, corr_o, ups_o, s));
   }
   if (host_ups) CK(cudaMemcpyAsync(upsilon, d_ups, ups_bytes * n_out, cudaMemcpyDeviceToHost, s));
   if (host_xi) CK(cudaMemcpyAsync(xi_acc, d_xi, xi_bytes * n_out, cudaMemcpyDeviceToHost, s));

@@ -59,71 +59,143 @@ __device__ __forceinline__ void order2(int& k0, int& b0, int& k1, int& b1) {
 
 // Block = (component, n2, n3): its nb^3 values come from one or a few rows (sg, a) of the
 // reduced array (nb npairs complex each), which stay in the cache, and are added into one
-// contiguous stretch of the output.
+// contiguous stretch of the output, less the multiple-counting terms where two bins are the same:
+// one nb x nb matrix for each pair of factors that can merge, staged in shared memory.  The output's
+// read and write bound it, and the FP64 additions next (16 clocks a warp instruction and SM).
+// n_max = 20, 10 bins (242 MB of output): 199 us, expansion and corrections as two kernels 491 us.
+constexpr int kExpandThreads = 256, kExpandValues = 4;
 template <bool SLICES>
-__global__ void __launch_bounds__(256) expand_kernel(const __grid_constant__ Basis B, const double2* __restrict__ red,
-                                                     int slices, double2* __restrict__ ups) {
-  const int N = B.N, nb = B.nb, nn = 2 * N + 1, np = B.npairs;
+__global__ void __launch_bounds__(kExpandThreads) expand_kernel(const __grid_constant__ Basis B,
+                                                                const double2* __restrict__ red, int slices,
+                                                                const double2* __restrict__ corr, int inv,
+                                                                double2* __restrict__ ups) {
+  extern __shared__ double2 merged[];  // [3][nb][nb]: factors (1, 2), (1, 3), (2, 3); triple [nb]
+  const int N = B.N, nb = B.nb, np = B.npairs, nn = 2 * N + 1, nb2 = nb * nb, nb3 = nb2 * nb;
   const int mu = blockIdx.x / (nn * nn), n2 = (blockIdx.x / nn) % nn - N, n3 = blockIdx.x % nn - N, s = n2 + n3;
-  const bool odd = mu == 1 || mu >= 5;  // x^* at the centre: F1 or F3
   const size_t stride = B.elems();
-  double2* out = ups + (size_t)blockIdx.x * nb * nb * nb;
-  for (int e = threadIdx.x; e < nb * nb * nb; e += blockDim.x) {
-    const int b[3] = {e / (nb * nb), (e / nb) % nb, e % nb};
-    size_t at;
-    double sign = 1.0;
-    if (mu == 8) {
-      const bool flip = s < 0;  // FW[-sg, -a] = FW[sg, a]^*
-      int k2 = flip ? n2 : -n2, k3 = flip ? n3 : -n3, c2 = b[1], c3 = b[2];
-      order2(k2, c2, k3, c3);
-      const int as = flip ? -s : s;
-      const size_t row = (size_t)(B.wbase(as) + k2 + N);
-      at = B.woff() + (row * nb + b[0]) * np + c2 * nb - c2 * (c2 - 1) / 2 + (c3 - c2);
-      if (flip) sign = -1.0;
+  const bool odd = mu == 1 || (mu >= 5 && mu < 8);  // x^* at the centre: F1 or F3
+  const bool flip = mu == 8 && s < 0;               // FW[-sg, -a] = FW[sg, a]^*
+  // family, place of its column among the three factors, sg of that column (families F2, F3) and
+  // the multipole index of every factor
+  const int q = mu == 8 ? 4 : mu < 2 ? mu : odd ? 3 : 2;
+  const int place = mu == 3 || mu == 6 ? 1 : mu == 4 || mu == 7 ? 2 : 0;
+  int k[3];
+  k[0] = mu == 8 ? (flip ? -s : s) : odd ? s - 1 : s - 3;
+  k[1] = mu == 8 ? (flip ? n2 : -n2) : -n2 - 2;
+  k[2] = mu == 8 ? (flip ? n3 : -n3) : odd ? -n3 - 1 : -n3 - 3;
+  const int sgc = place == 0 ? (odd ? -s - 3 : -s - 5) : place == 1 ? (odd ? n2 - 2 : n2 - 6) : odd ? n3 - 3 : n3 - 5;
+  const CorrLayout C = CorrLayout::make(N, nb);
+  for (int i = threadIdx.x; i < 3 * nb2 + nb; i += kExpandThreads) {
+    double2 v;
+    if (i >= 3 * nb2) {
+      v = corr[C.ot + (size_t)q * nb + (i - 3 * nb2)];
     } else {
-      // the three (index, bin) pairs: the column's, then the row's two
-      int k0 = odd ? s - 1 : s - 3, k1 = -n2 - 2, k2 = odd ? -n3 - 1 : -n3 - 3;
-      int c0 = b[0], c1 = b[1], c2 = b[2], sg, q;
-      if (mu < 2) {
-        order2(k0, c0, k1, c1);
-        order2(k1, c1, k2, c2);
-        order2(k0, c0, k1, c1);
-        sg = (mu ? -4 : -8) - k0;
-        q = mu;
+      const int m = i / nb2, third = 2 - m;  // pairs (0, 1), (0, 2), (1, 2) leave factor 2, 1, 0
+      const int c = third == 2 ? k[2] : third == 1 ? k[1] : k[0];
+      size_t at;
+      if (q == 4) {
+        at = C.ow + (size_t)(c < 0 ? -c : c) * nb2;
+      } else if (q >= 2 && third == place) {  // both row factors merged: the third is the column
+        at = (size_t)(q == 2 ? 2 : 4) * C.nsig * nb2 + (size_t)(sgc + 2 * N + 6) * nb2;
       } else {
-        // the conjugated factor is the column's: its place is bin 1, 2 or 3
-        const int place = (mu == 2 || mu == 5) ? 0 : (mu == 3 || mu == 6) ? 1 : 2;
-        if (place == 0) sg = odd ? -s - 3 : -s - 5;
-        else if (place == 1) { sg = odd ? n2 - 2 : n2 - 6; k1 = k0; c1 = c0; c0 = b[1]; }
-        else { sg = odd ? n3 - 3 : n3 - 5; k2 = k0; c2 = c0; c0 = b[2]; }
-        order2(k1, c1, k2, c2);
-        q = odd ? 3 : 2;
+        at = (size_t)(q < 2 ? q : q == 2 ? 3 : 5) * C.nsig * nb2 + (size_t)(2 * N + 6 - c - (odd ? 4 : 8)) * nb2;
       }
-      const int si = sg - B.sg0;
-      const size_t row = (size_t)(B.xbase[si] + k1 - B.xlo[si]);
-      at = (row * 4 * nb + q * nb + c0) * np + c1 * nb - c1 * (c1 - 1) / 2 + (c2 - c1);
+      v = corr[at + (i - m * nb2)];
+      if (q == 4 && c < 0) v.y = -v.y;
     }
+    merged[i] = v;
+  }
+  __syncthreads();
+  // (all three bins the same: the three terms less twice the triple one, at the first matrix' diagonal)
+  if ((int)threadIdx.x < nb) {
+    const int i = threadIdx.x * (nb + 1);
+    const double2 t = merged[3 * nb2 + threadIdx.x], m1 = merged[nb2 + i], m2 = merged[2 * nb2 + i];
+    merged[i].x += m1.x + m2.x - 2.0 * t.x;
+    merged[i].y += m1.y + m2.y - 2.0 * t.y;
+  }
+  __syncthreads();
+  double2* out = ups + (size_t)blockIdx.x * nb3;
+  // the reduced array's value of the triple (b0, b1, b2)
+  auto value = [&](int b0, int b1, int b2) -> double2 {
+    if (!red) return make_double2(0.0, 0.0);
+    int k0 = k[0], k1 = k[1], k2 = k[2], c0 = b0, c1 = b1, c2 = b2, sg = sgc;
+    if (q < 2) {  // any order of the three
+      order2(k0, c0, k1, c1);
+      order2(k1, c1, k2, c2);
+      order2(k0, c0, k1, c1);
+      sg = (q ? -4 : -8) - k0;
+    } else if (q == 4) {
+      order2(k1, c1, k2, c2);
+    } else {
+      if (place == 1) { k1 = k0; c1 = c0; c0 = b1; }
+      else if (place == 2) { k2 = k0; c2 = c0; c0 = b2; }
+      order2(k1, c1, k2, c2);
+    }
+    size_t at;
+    if (q == 4) at = B.woff() + ((size_t)(B.wbase(k0) + k1 + N) * nb + c0) * np;
+    else at = ((size_t)(B.xbase[sg - B.sg0] + k1 - B.xlo[sg - B.sg0]) * 4 * nb + q * nb + c0) * np;
+    at += c1 * nb - c1 * (c1 - 1) / 2 + (c2 - c1);
     double2 v = red[at];
     for (int z = 1; SLICES && z < slices; ++z) {
-      const double2 t = red[at + z * stride];
-      v.x += t.x;
-      v.y += t.y;
+      const double2 a = red[at + z * stride];
+      v.x += a.x;
+      v.y += a.y;
     }
-    double2 u = out[e];
-    u.x += v.x;
-    u.y += sign * v.y;
-    out[e] = u;
+    return v;
+  };
+  auto flipped = [&](double y) { return flip ? -y : y; };
+  // three different bins: nothing to take off
+  for (int e0 = threadIdx.x; e0 < nb3 && red; e0 += kExpandThreads * kExpandValues) {
+    double2 v[kExpandValues], u[kExpandValues];
+    bool use[kExpandValues];
+#pragma unroll
+    for (int i = 0; i < kExpandValues; ++i) {
+      const int e = e0 + i * kExpandThreads;
+      const int d = (e * inv) >> 20, b2 = e - d * nb, b0 = (d * inv) >> 20, b1 = d - b0 * nb;
+      use[i] = e < nb3 && b0 != b1 && b0 != b2 && b1 != b2;
+      if (use[i]) {
+        u[i] = out[e];
+        v[i] = value(b0, b1, b2);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kExpandValues; ++i)
+      if (use[i]) out[e0 + i * kExpandThreads] = make_double2(u[i].x + v[i].x, u[i].y + flipped(v[i].y));
+  }
+  // two or three the same: the nb (3 nb - 2) others, each with the term of its equal pair (they get
+  // lanes of their own: a predicated FP64 instruction takes its turn in the pipe whether it runs or not)
+  for (int i = threadIdx.x; i < nb * (3 * nb - 2); i += kExpandThreads) {
+    int m = 0, bm, bo;
+    if (i < nb2) {
+      bm = i / nb;
+      bo = i - bm * nb;
+    } else {
+      const int j = i - nb2, w = nb * (nb - 1), r = j % (nb - 1);
+      m = 1 + j / w;
+      bm = (j % w) / (nb - 1);
+      bo = r + (r >= bm);
+    }
+    const int b0 = m == 2 ? bo : bm, b1 = m == 1 ? bo : bm, b2 = m == 0 ? bo : bm;
+    const size_t e = ((size_t)b0 * nb + b1) * nb + b2;
+    const double2 u = out[e], v = value(b0, b1, b2), t = merged[m * nb2 + bm * nb + bo];
+    out[e] = make_double2(u.x + (v.x - t.x), u.y + flipped(v.y - t.y));
   }
 }
 
 }  // namespace
 
-cudaError_t basis_expand(const Basis& B, const double* red, int slices, double* ups, cudaStream_t s) {
-  const int nn = 2 * B.N + 1;
+cudaError_t basis_expand(const Basis& B, const double* red, int slices, const double* corr, double* ups,
+                         cudaStream_t s) {
+  const int nn = 2 * B.N + 1, blocks = 9 * nn * nn;
+  const int inv = ((1 << 20) + B.nb - 1) / B.nb;  // e / nb = (e inv) >> 20 for e < 32768, nb <= 32
   const double2* r = reinterpret_cast<const double2*>(red);
+  const double2* c = reinterpret_cast<const double2*>(corr);
   double2* u = reinterpret_cast<double2*>(ups);
-  if (slices > 1) expand_kernel<true><<<9 * nn * nn, 256, 0, s>>>(B, r, slices, u);
-  else expand_kernel<false><<<9 * nn * nn, 256, 0, s>>>(B, r, 1, u);
+  const size_t smem = (size_t)(3 * B.nb * B.nb + B.nb) * sizeof(double2);
+  auto kernel = slices > 1 ? expand_kernel<true> : expand_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<blocks, kExpandThreads, smem, s>>>(B, r, slices, c, inv, u);
   ++g_launches;
   return cudaGetLastError();
 }

@@ -66,9 +66,37 @@ __device__ __forceinline__ void basis_pair(int p, int nb, int& b2, int& b3) {
   b3 = b + (p - first);
 }
 
+// Sums of the multiple-counting terms (two or three of a quadruplet's neighbours the same galaxy; App.
+// A.1, Table tab:4PCFMCCorr).  Merging two factors of a family leaves the bin sum of their
+// per-galaxy product (XX, XA or WW of the record) times the third factor, so the terms of every
+// component come from seven arrays (bm: the merged pair's bin, bo: the third factor's):
+//   0: sum x   XX_sg(bm) G_{-sg-8}(bo)     F0, any two      1: sum x^* XX_sg(bm) G_{-sg-4}(bo)  F1, any two
+//   2: sum x   XX_sg(bm) G_{sg+4}^*(bo)    F2, rows merged  3: sum x   XA_{sg+4}(bm) G_{-sg-8}(bo)  F2, column merged
+//   4: sum x^* XX_sg(bm) G_sg^*(bo)        F3, rows merged  5: sum x^* XA_{sg+4}(bm) G_{-sg-4}(bo)  F3, column merged
+//   6: sum w   WW_c^*(bm) W_c(bo), c >= 0  FW, any two
+// and five triple sums.  Layout of a copy, complex: [6][nsig][nb][nb] (sg = -2N-6 + i), [2N+1][nb][nb],
+// triple [5][nb], xi accumulators [3][nb].
+struct CorrLayout {
+  int N, nb, nsig;
+  size_t ow, ot, ox, elems;
+  __host__ __device__ static CorrLayout make(int N, int nb) {
+    CorrLayout c;
+    c.N = N;
+    c.nb = nb;
+    c.nsig = 4 * N + 5;
+    c.ow = (size_t)6 * c.nsig * nb * nb;
+    c.ot = c.ow + (size_t)(2 * N + 1) * nb * nb;
+    c.ox = c.ot + (size_t)5 * nb;
+    c.elems = c.ox + (size_t)3 * nb;
+    return c;
+  }
+};
+
 // every ordered triple of bins at |n| <= N from the reduced array (the sum of `slices` arrays, one
-// after the other), added into ups
-cudaError_t basis_expand(const Basis& B, const double* red, int slices, double* ups, cudaStream_t s);
+// after the other; none if red is null) less the multiple-counting terms of the slot's first copy of
+// correction sums, added into ups
+cudaError_t basis_expand(const Basis& B, const double* red, int slices, const double* corr, double* ups,
+                         cudaStream_t s);
 
 // contract.cu: reduced arrays (slices of a wave's centres) of the CUDA-core contraction
 int contract_slices(const Basis& B);

@@ -243,13 +243,16 @@ struct Basis;
 template <typename R>
 cudaError_t contract_wave(const Layout& L, const Basis& B, const cplx_t<R>* rec, const cplx_t<R>* xw, int T,
                           const int* n_live, int w0, double* red, cudaStream_t s);
-// correction sums of every segment into its slot: corr + slot * corrections_size(L), and
-// (xi_acc non-null) xi_acc + slot * 6 nb
+
+// corrections.cu: the multiple-counting sums (and xi accumulators) of every segment into its slot's
+// copies, corr + slot * corrections_slot_doubles; finish adds the copies of `count` slots into the
+// first one each and their xi sums into xi [n_out][nb][3][2] (if non-null)
 template <typename R>
-cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t<R>* xw, const WavePlan& plan,
-                             double* corr, double* xi_acc, cudaStream_t s);
-cudaError_t corrections_apply(const Layout& L, const double* corr, double* ups, cudaStream_t s);
-size_t corrections_size(const Layout& L);  // doubles
+cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t<R>* xw, const WavePlan& plan, int n_out,
+                             double* corr, bool xi, cudaStream_t s);
+cudaError_t corrections_finish(const Layout& L, int n_out, int first, int count, double* corr, double* xi,
+                               cudaStream_t s);
+size_t corrections_slot_doubles(const Layout& L, int n_out);
 
 // contract_tc.cu (tensor cores).  The wave is contracted into the reduced array of the
 // Theta2 <-> Theta3 symmetry (tc_reduced_doubles doubles, zeroed per catalogue); tc_expand adds
