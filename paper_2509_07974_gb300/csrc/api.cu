@@ -21,7 +21,10 @@ size_t real_space_smem(int N, int nphi);
 int map4_nsplit(int chunk_tri, int ntri, int n_ap);
 cudaError_t map4_partials(const double* ups, const double* edges_host, int nb, int N, int nphi,
                           const double* ap_host, int n_ap, double* E_scratch, double* norm_chunk,
-                          double* gam_chunk, int chunk_tri, int nsplit, double* partial, cudaStream_t s);
+                          double* gam_chunk, double* tables, int chunk_tri, int nsplit, double* partial,
+                          cudaStream_t s);
+size_t map4_table_bytes(int chunk_tri, int nphi, int n_ap);
+int map4_chunk(int ntri, int nphi, int n_ap);
 cudaError_t map4_finish_launch(const double* partial, int ntri, int n_ap, const double* d_xipm,
                                const double* d_tb, const double* d_area, int nb, const double* d_ap,
                                double* d_m4, double* d_eb, double* d_disc, cudaStream_t s);
@@ -120,7 +123,7 @@ struct ext4pcf_ctx {
   // waves
   DBuf centres, flags, rec, xw, corr, counter, ncen;
   // transforms
-  DBuf t_norm, t_gam, t_E, t_part, t_small;
+  DBuf t_norm, t_gam, t_E, t_tab, t_part, t_small;
   // direct aperture estimator: centres, per-split sums, staged outputs
   DBuf ap_cen, ap_sums, io_rec, io_mom;
   // tensor-core contraction: work items (built once per shape) and the device status word
@@ -270,7 +273,7 @@ int ext4pcf_destroy(ext4pcf_ctx* ctx) {
                  &ctx->keys, &ctx->keys_alt, &ctx->perm, &ctx->perm_alt, &ctx->cell_start, &ctx->hist,
                  &ctx->px, &ctx->py, &ctx->xr, &ctx->xi, &ctx->w, &ctx->p4, &ctx->s4, &ctx->bbox,
                  &ctx->centres, &ctx->flags, &ctx->rec, &ctx->xw, &ctx->corr, &ctx->counter, &ctx->ncen,
-                 &ctx->t_norm, &ctx->t_gam, &ctx->t_E, &ctx->t_part, &ctx->t_small, &ctx->tc_items,
+                 &ctx->t_norm, &ctx->t_gam, &ctx->t_E, &ctx->t_tab, &ctx->t_part, &ctx->t_small, &ctx->tc_items,
                  &ctx->tc_xb, &ctx->tc_red, &ctx->tc_rowmax, &ctx->status, &ctx->geom, &ctx->ap_cen, &ctx->ap_sums, &ctx->io_rec, &ctx->io_mom};
   for (DBuf* b : all)
     if (b->p) cudaFree(b->p);
@@ -1081,11 +1084,11 @@ int ext4pcf_to_map4(ext4pcf_ctx* ctx, const double* upsilon, const double* radia
   cudaStream_t s = ctx->stream;
   const int ntri = n_bins * n_bins * n_bins;
   const size_t nph2 = (size_t)n_phi * n_phi;
-  int chunk = (int)std::max<size_t>(1, (size_t)(256u << 20) / (nph2 * 8 * 16));
-  if (chunk > ntri) chunk = ntri;
+  const int chunk = map4_chunk(ntri, n_phi, n_ap);
   ENSURE(ctx->t_norm, (size_t)chunk * nph2 * 8);
   ENSURE(ctx->t_gam, (size_t)chunk * nph2 * 8 * 16);
   ENSURE(ctx->t_E, (size_t)(2 * n_max + 1) * n_phi * 16);
+  ENSURE(ctx->t_tab, map4_table_bytes(chunk, n_phi, n_ap));
   const int nsplit = map4_nsplit(chunk, ntri, n_ap);
   ENSURE(ctx->t_part, (size_t)ntri * nsplit * n_ap * 8 * 16);
   // small buffer: xi_acc [nb*6], tb [nb], area [nb], ap [n_ap], m4 [n_ap*16], eb [n_ap*16], disc [n_ap*16]
@@ -1107,7 +1110,7 @@ int ext4pcf_to_map4(ext4pcf_ctx* ctx, const double* upsilon, const double* radia
     CK(cudaMemcpyAsync(d_small, xi_acc, (size_t)n_bins * 6 * 8,
                        is_device_ptr(xi_acc) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   CK(map4_partials(upsilon, radial_bins, n_bins, n_max, n_phi, ap_radii, n_ap, (double*)ctx->t_E.p,
-                   (double*)ctx->t_norm.p, (double*)ctx->t_gam.p, chunk, nsplit, (double*)ctx->t_part.p, s));
+                   (double*)ctx->t_norm.p, (double*)ctx->t_gam.p, (double*)ctx->t_tab.p, chunk, nsplit, (double*)ctx->t_part.p, s));
   double* d_m4 = d_small + 8 * n_bins + n_ap;
   double* d_eb = d_m4 + 16 * n_ap;
   double* d_disc = d_eb + 16 * n_ap;

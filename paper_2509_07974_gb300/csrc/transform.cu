@@ -10,6 +10,7 @@
 //      J_mu = sum_p P_p R_p pi p! (theta^2/2)^{p+1},
 //    P(z^*) = prod over unconjugated apertures (z^* + d_a^*)^2, R(z) = prod over conjugated
 //    apertures (z + d_a)^2, ph_mu = 2 sum_a s_a zeta_a of the x-projection (s = +-1).
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -42,53 +43,112 @@ __global__ void angle_table(int N, int nphi, double2* E) {
   }
 }
 
-// Bin counts of component mu for radial triples [tri0, tri0 + gridDim.x / ncomp).
-// IS_NORM: writes real N counts to out_norm[tri][p][q]; otherwise writes
-// Upsilon / N to out_gam[mu][tri][p][q] (complex, accumulated), reading norm.
-template <bool IS_NORM>
-__global__ void real_space_kernel(const double2* __restrict__ ups, int nb, int N, int nphi,
-                                  const double2* __restrict__ E, int tri0, int ntri,
-                                  const double* __restrict__ norm_in, double* __restrict__ norm_out,
-                                  double2* __restrict__ gam_out, size_t gam_mu_stride) {
+// What real_space_kernel writes: the angular-bin counts of the normalisation, their reciprocals (see
+// recip_of), Upsilon / N added into gamma, or Upsilon times the reciprocals of N.
+enum RealOut { kCounts, kRecips, kGammaAdd, kGammaTimes };
+
+// One reciprocal per angular bin serves the eight components (a division is ten FP64 operations).  A
+// count whose reciprocal could leave the normal range, 0, infinities and NaN stay as they are: the
+// magnitude tells the two apart.
+constexpr double kRecipMax = 0x1p960, kRecipMin = 0x1p-960;
+__device__ __forceinline__ bool is_recip(double v) { return fabs(v) >= kRecipMin && fabs(v) <= kRecipMax; }
+__device__ __forceinline__ double recip_of(double count) { return is_recip(count) ? 1.0 / count : count; }
+
+// One block per (component, radial triple): the separable sum over n3, then n2, of
+// Upsilon_n E_n2(p) E_n3(q).  E_-n = E_n^*, and the bin p' = n_phi - 1 - p mirrors p: E_n(p') =
+// E_n(p)^*.  With A_n = u_n + u_-n and B_n = u_n - u_-n a sum over n is
+//   u_0 E_0 + sum_{n>0} A_n Re E_n(p) + i B_n Im E_n(p)   at p, and with - i at p':
+// four FP64 multiply-adds for two n at two bins where the plain sum takes sixteen.  The FP64 pipe (2
+// multiply-adds per clock and SM) bounds it; shared memory and the table are far from their limits,
+// so a thread simply owns one (row or bin q, bin p) at a time.  1000 triples, n_max = 20, 129
+// angular bins, nine components: 95 -> 15.6 ms.
+constexpr int kRealThreads = 512;
+template <RealOut OUT>
+__global__ void __launch_bounds__(kRealThreads, 2)
+real_space_kernel(const double2* __restrict__ ups, int nb, int N, int nphi, const double2* __restrict__ E, int tri0,
+                  int ntri, const double* __restrict__ norm_in, double* __restrict__ norm_out,
+                  double2* __restrict__ gam_out, size_t gam_mu_stride) {
+  constexpr bool kNorm = OUT == kCounts || OUT == kRecips;
   extern __shared__ double2 sm[];
-  const int nn = 2 * N + 1;
-  const int mu = IS_NORM ? 8 : (int)(blockIdx.x / ntri);
+  const int nn = 2 * N + 1, half = (nphi + 1) / 2;
+  const int mu = kNorm ? 8 : (int)(blockIdx.x / ntri);
   const int lt = (int)(blockIdx.x % ntri), tri = tri0 + lt;
   const size_t nb3 = (size_t)nb * nb * nb;
   double2* U = sm;                 // [nn][nn]
   double2* T1 = sm + nn * nn;      // [nn][nphi]
-  for (int k = threadIdx.x; k < nn * nn; k += blockDim.x) {
-    const int a2 = k / nn, a3 = k % nn;
-    U[k] = ups[(((size_t)mu * nn + a2) * nn + a3) * nb3 + tri];
+  for (int k = threadIdx.x; k < nn * nn; k += blockDim.x) U[k] = ups[((size_t)mu * nn * nn + k) * nb3 + tri];
+  __syncthreads();
+  // (A_n, B_n) in the places of (u_n, u_-n)
+  for (int k = threadIdx.x; k < nn * N; k += blockDim.x) {
+    double2& hi = U[(k / N) * nn + N + 1 + k % N];
+    double2& lo = U[(k / N) * nn + N - 1 - k % N];
+    const double2 u = hi, v = lo;
+    hi = make_double2(u.x + v.x, u.y + v.y);
+    lo = make_double2(u.x - v.x, u.y - v.y);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < nn * nphi; k += blockDim.x) {
-    const int a2 = k / nphi, q = k % nphi;
-    double re = 0, im = 0;
-    for (int a3 = 0; a3 < nn; ++a3) {
-      const double2 u = U[a2 * nn + a3], e = E[a3 * nphi + q];
-      re += u.x * e.x - u.y * e.y;
-      im += u.x * e.y + u.y * e.x;
+  const double e0 = 1.0 / nphi;  // E_0
+  for (int k = threadIdx.x; k < nn * half; k += blockDim.x) {
+    const int a2 = k / half, q = k - a2 * half;
+    const double2* u = U + a2 * nn + N;
+    double sx = u[0].x * e0, sy = u[0].y * e0, dx = 0, dy = 0;
+    for (int n = 1; n <= N; ++n) {
+      const double2 e = E[(N + n) * nphi + q], A = u[n], B = u[-n];
+      sx += A.x * e.x;
+      sy += A.y * e.x;
+      dx += B.x * e.y;
+      dy += B.y * e.y;
     }
-    T1[k] = make_double2(re, im);
+    T1[a2 * nphi + q] = make_double2(sx - dy, sy + dx);
+    if (q != nphi - 1 - q) T1[a2 * nphi + nphi - 1 - q] = make_double2(sx + dy, sy - dx);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < N * nphi; k += blockDim.x) {
+    const int n = 1 + k / nphi, q = k % nphi;
+    double2& hi = T1[(N + n) * nphi + q];
+    double2& lo = T1[(N - n) * nphi + q];
+    const double2 u = hi, v = lo;
+    hi = make_double2(u.x + v.x, u.y + v.y);
+    lo = make_double2(u.x - v.x, u.y - v.y);
   }
   __syncthreads();
   const size_t nph2 = (size_t)nphi * nphi;
-  for (int k = threadIdx.x; k < nphi * nphi; k += blockDim.x) {
-    const int p = k / nphi, q = k % nphi;
-    double re = 0, im = 0;
-    for (int a2 = 0; a2 < nn; ++a2) {
-      const double2 e = E[a2 * nphi + p], t = T1[a2 * nphi + q];
-      re += e.x * t.x - e.y * t.y;
-      im += e.x * t.y + e.y * t.x;
+  for (int k = threadIdx.x; k < half * nphi; k += blockDim.x) {
+    const int p = k / nphi, q = k - p * nphi;
+    const double2* t = T1 + N * nphi + q;
+    double sx = t[0].x * e0, sy = t[0].y * e0, dx = 0, dy = 0;
+    for (int n = 1; n <= N; ++n) {
+      const double2 e = E[(N + n) * nphi + p], A = t[n * nphi], B = t[-n * nphi];
+      sx += A.x * e.x;
+      dy += B.y * e.y;
+      if (!kNorm) {
+        sy += A.y * e.x;
+        dx += B.x * e.y;
+      }
     }
-    const size_t o = (size_t)lt * nph2 + k;
-    if (IS_NORM) {
-      norm_out[o] = re;
-    } else {
-      const double nv = norm_in[o];
-      double2& g = gam_out[(size_t)mu * gam_mu_stride + o];
-      if (nv != 0.0) { g.x += re / nv; g.y += im / nv; }
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {  // p, and its mirror
+      const int pm = m ? nphi - 1 - p : p;
+      if (m && pm == p) break;
+      const double re = m ? sx + dy : sx - dy, im = m ? sy - dx : sy + dx;
+      const size_t o = (size_t)lt * nph2 + (size_t)pm * nphi + q;
+      if (OUT == kCounts) {
+        norm_out[o] = re;
+      } else if (OUT == kRecips) {
+        norm_out[o] = recip_of(re);
+      } else {
+        const double nv = norm_in[o];
+        double2* g = gam_out + (size_t)mu * gam_mu_stride + o;
+        if (OUT == kGammaTimes) {
+          *g = is_recip(nv) ? make_double2(re * nv, im * nv)
+                            : nv != 0.0 ? make_double2(re / nv, im / nv) : make_double2(0, 0);
+        } else if (nv != 0.0) {
+          double2 v = *g;
+          v.x += re / nv;
+          v.y += im / nv;
+          *g = v;
+        }
+      }
     }
   }
 }
@@ -112,134 +172,209 @@ __device__ __forceinline__ double2 cm(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// block = (triple in chunk, slice of the angular bins).  The aperture-independent part of
-// F_mu (Gamma_mu times the phase and geometric factors times the coefficients P_t R_t of
-// J_mu) is formed once per angular bin, kM4Bins bins at a time, and kept in shared memory;
-// then the threads, one per (mu, aperture) pair, fold the tile into their sums.  Only
-// t <= min(deg P, deg R) contributes: 0 for mu = 0, 2 for one conjugated aperture, 4 for two.
-constexpr int kM4Bins = 16;     // angular bins per tile (kM4Bins * 8 = blockDim items)
-constexpr int kM4Threads = 128;
-constexpr int kM4MaxPairs = 4;  // (mu, aperture) pairs per thread: 8 * 64 / 128
+// e^{-sum|d|^2 / 2 theta^2} is a product of three functions of one angle each: with
+// sum|d|^2 = (3/4) sum t^2 - (1/2) (t1 t2 cos p12 + t1 t3 cos p13 + t2 t3 cos(p12 - p13)) and
+// cos = 1 - 2 sin^2(./2) every exponent stays <= 0.  Tables [triple][3][nphi][n_ap], the constant
+// factor in the first; the third by (p - q) mod nphi: 3 nphi exponentials a radius, not nphi^2.
+__global__ void map4_tables(const Map4Args a, double* __restrict__ tab) {
+  const int per = 3 * a.nphi * a.n_ap;
+  const int lt = blockIdx.x, tri = a.tri0 + lt, nb = a.nb;
+  const double t1 = a.tb[tri / (nb * nb)], t2 = a.tb[(tri / nb) % nb], t3 = a.tb[tri % nb];
+  const double dphi = 2.0 * kPi / a.nphi;
+  const double base = 0.75 * (t1 * t1 + t2 * t2 + t3 * t3) - 0.5 * (t1 * t2 + t1 * t3 + t2 * t3);
+  for (int k = threadIdx.x; k < per; k += blockDim.x) {
+    const int w = k / (a.nphi * a.n_ap), p = (k / a.n_ap) % a.nphi, ia = k % a.n_ap;
+    const double sh = sin(0.5 * (w == 2 ? p : p + 0.5) * dphi);
+    const double tt = w == 0 ? t1 * t2 : w == 1 ? t1 * t3 : t2 * t3;
+    const double x = tt * sh * sh + (w == 0 ? base : 0.0);
+    const double th = a.ap[ia];
+    tab[(size_t)lt * per + k] = exp(-x / (2.0 * th * th));
+  }
+}
 
-__global__ void __launch_bounds__(kM4Threads) map4_kernel(const Map4Args a, const double2* __restrict__ gam,
-                                                          size_t gam_mu_stride, int nsplit,
+// e^{i phi} at the middle of every angular bin
+__global__ void map4_turns(int nphi, double2* __restrict__ turn) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= nphi) return;
+  double sn, cs;
+  sincos((p + 0.5) * (2.0 * kPi / nphi), &sn, &cs);
+  turn[p] = make_double2(cs, sn);
+}
+
+// The aperture integral of one radial triple over a slice of the angular bins.  The integrand is
+// Gamma_mu times C_{mu,t} = geo e^{i ph_mu} P_t R_t (t <= min(deg P, deg R): 0 for mu = 0, 2 for one
+// conjugated aperture, 4 for two: 28 coefficients) times the exponential and, at the end, the
+// radius' factor of t.  Mirroring both angles conjugates the d_a and so every C, and leaves the
+// exponential: the bins k and n_phi^2 - 1 - k are taken together,
+//   Gamma C + Gamma' C^* = (Gamma + Gamma') Re C + i (Gamma - Gamma') Im C.
+// Tiles of kM4Bins such pairs: one thread a pair forms all 28 coefficients (the products of the
+// d_a shared by the components; sum d_a = 0 gives half of them), then a thread per coefficient and
+// group of radii folds the tile into its sums.  FP64 multiply-adds bound it: 56 a pair and radius
+// for the sums, about 500 a pair for the coefficients.  1000 triples, 129 angular bins, 24 radii:
+// 198 -> 29.3 ms.
+constexpr int kM4Bins = 128;    // bin pairs per tile
+constexpr int kM4Row = kM4Bins + 1;  // a column of coefficients falls on different banks
+constexpr int kM4Coef = 28;     // (mu, t)
+constexpr int kM4Groups = 8;    // threads per coefficient
+constexpr int kM4Threads = kM4Coef * kM4Groups;
+constexpr int kM4Radii = 8;     // radii per thread: 64 / kM4Groups
+// first coefficient of component mu
+__host__ __device__ constexpr int m4_first(int mu) { return mu == 0 ? 0 : mu < 5 ? 1 + 3 * (mu - 1) : 13 + 5 * (mu - 5); }
+static_assert(m4_first(8) == kM4Coef, "coefficients");
+
+__device__ __forceinline__ double2 conj2(double2 a) { return make_double2(a.x, -a.y); }
+__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 sc2(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
+
+__global__ void __launch_bounds__(kM4Threads, 2) map4_kernel(const Map4Args a, const double2* __restrict__ gam,
+                                                          size_t gam_mu_stride, const double* __restrict__ tab,
+                                                          const double2* __restrict__ turn, int nsplit,
                                                           double2* __restrict__ partial) {
-  __shared__ double2 coef[kM4Bins][8][5];  // Gamma_mu e^{i ph_mu} geo P_t R_t, t <= 4
-  __shared__ double exs[kM4Bins][64];      // e^{-sum|d|^2 / 2 theta^2} per bin and aperture
-  __shared__ double sd2s[kM4Bins];
-  __shared__ double hps[64][5];            // pi t! h^{t+1} / (4 pi theta^4)^4
-  const size_t nph2 = (size_t)a.nphi * a.nphi;
-  const int lt = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
-  const int tri = a.tri0 + lt, nb = a.nb;
+  extern __shared__ double2 m4s[];
+  double2* coef = m4s;                                             // [kM4Coef][kM4Row]
+  double* exs = reinterpret_cast<double*>(coef + kM4Coef * kM4Row);  // [n_ap][kM4Bins]
+  const int nphi = a.nphi, n_ap = a.n_ap, nb = a.nb, tid = threadIdx.x;
+  const long long nph2 = (long long)nphi * nphi, halfn = (nph2 + 1) / 2;
+  const int lt = blockIdx.x / nsplit, split = blockIdx.x % nsplit, tri = a.tri0 + lt;
   const int b1 = tri / (nb * nb), b2 = (tri / nb) % nb, b3 = tri % nb;
   const double t1 = a.tb[b1], t2 = a.tb[b2], t3 = a.tb[b3];
-  const double dphi = 2.0 * kPi / a.nphi;
+  const double dphi = 2.0 * kPi / nphi;
   const double geo = 2.0 * kPi * t1 * t2 * t3 * a.vol[b1] * a.vol[b2] * a.vol[b3] * dphi * dphi;
-  const size_t kbeg = nph2 * split / nsplit, kend = nph2 * (split + 1) / nsplit;
-  for (int ia = threadIdx.x; ia < a.n_ap; ia += blockDim.x) {
-    const double th2 = a.ap[ia] * a.ap[ia], h = 0.5 * th2;
-    const double q0 = 4.0 * kPi * th2 * th2;
-    const double norm = 1.0 / (q0 * q0 * q0 * q0);
-    double f = 1.0, hh = h;
-    for (int t = 0; t < 5; ++t) { if (t > 0) f *= t; hps[ia][t] = kPi * f * hh * norm; hh *= h; }
-  }
-  const int npairs = 8 * a.n_ap;
-  double2 acc[kM4MaxPairs];
-  for (int r = 0; r < kM4MaxPairs; ++r) acc[r] = make_double2(0, 0);
-  for (size_t k0 = kbeg; k0 < kend; k0 += kM4Bins) {
-    __syncthreads();  // previous tile fully consumed (and hps written)
-    {
-      // one (bin, mu) item per thread
-      const int j = threadIdx.x >> 3, mu = threadIdx.x & 7;
-      const size_t k = k0 + j;
-      if (k >= kend) {
-        for (int t = 0; t < 5; ++t) coef[j][mu][t] = make_double2(0, 0);
-        if (mu == 0) sd2s[j] = 0;
-      } else {
-        const int p = (int)(k / a.nphi), q = (int)(k % a.nphi);
-        const double p12 = (p + 0.5) * dphi, p13 = (q + 0.5) * dphi;
-        double s12, c12, s13, c13;
-        sincos(p12, &s12, &c12);
-        sincos(p13, &s13, &c13);
-        const double2 v[4] = {make_double2(0, 0), make_double2(t1, 0), make_double2(t2 * c12, t2 * s12),
-                              make_double2(t3 * c13, t3 * s13)};
-        const double2 cen =
-            make_double2((v[1].x + v[2].x + v[3].x) * 0.25, (v[1].y + v[2].y + v[3].y) * 0.25);
-        double2 d[4];
-        double sd2 = 0;
-        for (int jj = 0; jj < 4; ++jj) {
-          d[jj] = make_double2(v[jj].x - cen.x, v[jj].y - cen.y);
-          sd2 += d[jj].x * d[jj].x + d[jj].y * d[jj].y;
-        }
-        if (mu == 0) sd2s[j] = sd2;
-        double2 P[9], R[9];
-        int dP = 0, dR = 0;
-        P[0] = make_double2(1, 0);
-        R[0] = make_double2(1, 0);
-        for (int jj = 0; jj < 4; ++jj) {
-          const bool cj = kBeta[mu][jj];
-          double2* poly = cj ? R : P;
-          int& dg = cj ? dR : dP;
-          const double2 root = cj ? d[jj] : make_double2(d[jj].x, -d[jj].y);
-          for (int rep = 0; rep < 2; ++rep) {
-            poly[dg + 1] = poly[dg];
-            for (int t = dg; t >= 1; --t) {
-              const double2 m = cm(poly[t], root);
-              poly[t] = make_double2(poly[t - 1].x + m.x, poly[t - 1].y + m.y);
-            }
-            poly[0] = cm(poly[0], root);
-            ++dg;
-          }
-        }
-        // e^{i ph}, ph = 2 sum s_a zeta_a, zeta = (phi13/2, 0, phi12, phi13)
-        const double ph = (kBeta[mu][0] ? -1.0 : 1.0) * p13 + 2.0 * (kBeta[mu][2] ? -1.0 : 1.0) * p12 +
-                          2.0 * (kBeta[mu][3] ? -1.0 : 1.0) * p13;
-        double sp, cp;
-        sincos(ph, &sp, &cp);
-        const double2 g =
-            cm(gam[(size_t)mu * gam_mu_stride + (size_t)lt * nph2 + k], make_double2(cp * geo, sp * geo));
-        const int tmax = dP < dR ? dP : dR;
-        for (int t = 0; t < 5; ++t) coef[j][mu][t] = t <= tmax ? cm(g, cm(P[t], R[t])) : make_double2(0, 0);
+  const double* tb = tab + (size_t)lt * 3 * nphi * n_ap;
+  const long long kbeg = halfn * split / nsplit, kend = halfn * (split + 1) / nsplit;
+  // this thread's coefficient, radii and (few radii) part of every tile
+  const int c = tid % kM4Coef, grp = tid / kM4Coef;
+  const int lanes = min(kM4Groups, n_ap), parts = kM4Groups / lanes, part = grp / lanes, ia0 = grp % lanes;
+  const bool sums = part < parts;
+  double2 acc[kM4Radii];
+#pragma unroll
+  for (int r = 0; r < kM4Radii; ++r) acc[r] = make_double2(0, 0);
+  for (long long k0 = kbeg; k0 < kend; k0 += kM4Bins) {
+    const int nk = (int)min((long long)kM4Bins, kend - k0);
+    __syncthreads();  // the previous tile is done with
+    if (tid < nk) {
+      const long long k = k0 + tid, km = nph2 - 1 - k;
+      const int p = (int)(k / nphi), q = (int)(k % nphi);
+      const double2 e2 = turn[p], e3 = turn[q];
+      // the neighbours' places less a quarter of their sum: d_0 .. d_3, and their conjugates u_a
+      const double2 v2 = sc2(t2, e2), v3 = sc2(t3, e3);
+      const double2 cen = make_double2(0.25 * (t1 + v2.x + v3.x), 0.25 * (v2.y + v3.y));
+      const double2 d[4] = {make_double2(-cen.x, -cen.y), make_double2(t1 - cen.x, -cen.y),
+                            make_double2(v2.x - cen.x, v2.y - cen.y), make_double2(v3.x - cen.x, v3.y - cen.y)};
+      // products of two: q01 .. q23 of the d_a (those of the u_a are their conjugates)
+      const double2 q01 = cm(d[0], d[1]), q02 = cm(d[0], d[2]), q03 = cm(d[0], d[3]), q12 = cm(d[1], d[2]),
+                    q13 = cm(d[1], d[3]), q23 = cm(d[2], d[3]);
+      // phases e^{i ph_mu}, from e^{2 i p12}, e^{i p13}, e^{3 i p13}, with the geometric factor
+      const double2 e22 = sc2(geo, cm(e2, e2)), e33 = cm(cm(e3, e3), e3);
+      const double2 f23 = cm(e22, e33), f21 = cm(e22, e3), f2m1 = cm(e22, conj2(e3)), f2m3 = cm(e22, conj2(e33));
+      auto put = [&](int mu, int t, double2 C) {
+        // (Gamma + Gamma') Re C + i (Gamma - Gamma') Im C; the middle bin is its own mirror
+        const double2 g = gam[(size_t)mu * gam_mu_stride + (size_t)lt * nph2 + k];
+        const double2 h = km != k ? gam[(size_t)mu * gam_mu_stride + (size_t)lt * nph2 + km] : make_double2(0, 0);
+        const double sx = g.x + h.x, sy = g.y + h.y, dx = g.x - h.x, dy = g.y - h.y;
+        coef[(m4_first(mu) + t) * kM4Row + tid] = make_double2(sx * C.x - dy * C.y, sy * C.x + dx * C.y);
+      };
+      {  // mu = 0: (u_0 u_1 u_2 u_3)^2
+        const double2 P = conj2(cm(q01, q23));
+        put(0, 0, cm(f23, cm(P, P)));
       }
+      // one conjugated aperture c, the others' u: E_0 = their product, E_1 their products of two, E_2
+      // their sum = -u_c; P = (E_0^2, 2 E_0 E_1, E_1^2 + 2 E_0 E_2), R = (d_c^2, 2 d_c, 1)
+      auto one = [&](int mu, double2 dc, double2 pa, double2 pb, double2 pc, double2 third, double2 ph) {
+        const double2 E0 = conj2(cm(pa, third)), E1 = conj2(add2(add2(pa, pb), pc));
+        const double2 E0d = cm(E0, dc);
+        put(mu, 0, cm(ph, cm(E0d, E0d)));
+        put(mu, 1, sc2(4.0, cm(ph, cm(E0d, E1))));
+        const double2 w = cm(E0, conj2(dc)), s = cm(E1, E1);
+        put(mu, 2, cm(ph, make_double2(s.x - 2.0 * w.x, s.y - 2.0 * w.y)));
+      };
+      one(1, d[0], q12, q13, q23, d[3], f21);
+      one(2, d[1], q02, q03, q23, d[3], f23);
+      one(3, d[2], q01, q03, q13, d[3], conj2(f2m3));
+      one(4, d[3], q01, q02, q12, d[2], f2m1);
+      // two conjugated: p = u_a u_b, s = u_a + u_b, p' = d_c d_e, s' = d_c + d_e = -s^*:
+      // P R = (p p')^2, 4 p p' s s', (s^2 + 2 p)(s'^2 + 2 p'), 4 s s', 1
+      auto two = [&](int mu, double2 pu, double2 s, double2 pd, double2 ph) {
+        const double2 pp = cm(pu, pd);
+        const double ss = -(s.x * s.x + s.y * s.y);  // s s'
+        put(mu, 0, cm(ph, cm(pp, pp)));
+        put(mu, 1, sc2(4.0 * ss, cm(ph, pp)));
+        const double2 s2 = cm(s, s), x = make_double2(s2.x + 2.0 * pu.x, s2.y + 2.0 * pu.y),
+                      y = make_double2(s2.x + 2.0 * pd.x, -s2.y + 2.0 * pd.y);  // s'^2 = (s^2)^*
+        put(mu, 2, cm(ph, cm(x, y)));
+        put(mu, 3, sc2(4.0 * ss, ph));
+        put(mu, 4, ph);
+      };
+      two(5, conj2(q23), conj2(add2(d[2], d[3])), q01, f21);
+      two(6, conj2(q13), conj2(add2(d[1], d[3])), q02, conj2(f2m1));
+      two(7, conj2(q12), conj2(add2(d[1], d[2])), q03, f2m3);
+    }
+    // exponentials of the tile, zero past its end
+    for (int w = tid; w < kM4Bins * n_ap; w += kM4Threads) {
+      const int ia = w / kM4Bins, j = w % kM4Bins;
+      double e = 0.0;
+      if (j < nk) {
+        const long long k = k0 + j;
+        const int p = (int)(k / nphi), q = (int)(k % nphi), pq = p >= q ? p - q : p - q + nphi;
+        e = tb[p * n_ap + ia] * tb[(nphi + q) * n_ap + ia] * tb[(2 * nphi + pq) * n_ap + ia];
+      }
+      exs[ia * kM4Bins + j] = e;
     }
     __syncthreads();
-    for (int w = threadIdx.x; w < kM4Bins * a.n_ap; w += blockDim.x) {
-      const int j = w / a.n_ap, ia = w % a.n_ap;
-      const double th = a.ap[ia];
-      exs[j][ia] = exp(-sd2s[j] / (2.0 * th * th));
-    }
-    __syncthreads();
-    for (int r = 0; r < kM4MaxPairs; ++r) {
-      const int pr = threadIdx.x + r * kM4Threads;
-      if (pr >= npairs) break;
-      const int mu = pr / a.n_ap, ia = pr % a.n_ap;
-      const int tmax = mu == 0 ? 0 : (mu < 5 ? 2 : 4);
-      double2 s = acc[r];
-      for (int j = 0; j < kM4Bins; ++j) {
-        double re = 0, im = 0;
-        for (int t = 0; t <= tmax; ++t) {
-          re += coef[j][mu][t].x * hps[ia][t];
-          im += coef[j][mu][t].y * hps[ia][t];
+    if (sums) {
+      const int j0 = nk * part / parts, j1 = nk * (part + 1) / parts;
+#pragma unroll
+      for (int r = 0; r < kM4Radii; ++r) {
+        const int ia = ia0 + r * lanes;
+        if (ia >= n_ap) break;
+        double2 s = acc[r];
+        const double2* cf = coef + c * kM4Row;
+        const double* ex = exs + ia * kM4Bins;
+        for (int j = j0; j < j1; ++j) {
+          s.x += cf[j].x * ex[j];
+          s.y += cf[j].y * ex[j];
         }
-        s.x += re * exs[j][ia];
-        s.y += im * exs[j][ia];
+        acc[r] = s;
       }
-      acc[r] = s;
     }
   }
-  for (int r = 0; r < kM4MaxPairs; ++r) {
-    const int pr = threadIdx.x + r * kM4Threads;
-    if (pr >= npairs) break;
-    const int mu = pr / a.n_ap, ia = pr % a.n_ap;
-    partial[(((size_t)tri * nsplit + split) * a.n_ap + ia) * 8 + mu] = acc[r];
+  // the radius' factors pi t! h^{t+1} / (4 pi theta^4)^4, then the sum over t and parts
+  __syncthreads();
+  double2* tot = m4s;  // [parts][n_ap][kM4Coef]
+#pragma unroll
+  for (int r = 0; r < kM4Radii; ++r) {
+    const int ia = ia0 + r * lanes;
+    if (!sums || ia >= n_ap) break;
+    const int t = c == 0 ? 0 : c < 13 ? (c - 1) % 3 : (c - 13) % 5;
+    const double th2 = a.ap[ia] * a.ap[ia], h = 0.5 * th2, q0 = 4.0 * kPi * th2 * th2;
+    double f = kPi * h / (q0 * q0 * q0 * q0);
+    for (int i = 1; i <= t; ++i) f *= i * h;
+    tot[((size_t)part * n_ap + ia) * kM4Coef + c] = sc2(f, acc[r]);
+  }
+  __syncthreads();
+  for (int w = tid; w < 8 * n_ap; w += kM4Threads) {
+    const int ia = w / 8, mu = w % 8;
+    double2 s = make_double2(0, 0);
+    for (int pt = 0; pt < parts; ++pt)
+      for (int i = m4_first(mu); i < m4_first(mu + 1); ++i) s = add2(s, tot[((size_t)pt * n_ap + ia) * kM4Coef + i]);
+    partial[(((size_t)tri * nsplit + split) * n_ap + ia) * 8 + mu] = s;
   }
 }
 
 }  // namespace
 
-cudaError_t real_space_counts(const double* ups, int nb, int N, int nphi, double* E_scratch,
-                              int tri0, int ntri, double* norm_chunk, double* gam_chunk,
-                              size_t gam_mu_stride, bool accumulate_into_existing, cudaStream_t s);
+namespace {
+template <RealOut OUT>
+cudaError_t launch_real(int blocks, size_t smem, cudaStream_t s, const double2* U, int nb, int N, int nphi,
+                        const double2* E, int tri0, int ntri, const double* norm_in, double* norm_out, double2* gam,
+                        size_t stride) {
+  cudaError_t e = cudaFuncSetAttribute(real_space_kernel<OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  real_space_kernel<OUT><<<blocks, kRealThreads, smem, s>>>(U, nb, N, nphi, E, tri0, ntri, norm_in, norm_out, gam, stride);
+  ++g_launches;
+  return cudaGetLastError();
+}
+}  // namespace
 
 cudaError_t real_space(const double* ups, int nb, int N, int nphi, double* gamma, double* norm,
                        double* scratch_norm, double* E_scratch, cudaStream_t s) {
@@ -247,16 +382,14 @@ cudaError_t real_space(const double* ups, int nb, int N, int nphi, double* gamma
   const int ntri = nb * nb * nb;
   angle_table<<<64, 256, 0, s>>>(N, nphi, reinterpret_cast<double2*>(E_scratch));
   const size_t smem = (size_t)(nn * nn + nn * nphi) * sizeof(double2);
-  cudaError_t e = cudaFuncSetAttribute(real_space_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(real_space_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const double2* U = reinterpret_cast<const double2*>(ups);
   const double2* E = reinterpret_cast<const double2*>(E_scratch);
-  real_space_kernel<true><<<ntri, 256, smem, s>>>(U, nb, N, nphi, E, 0, ntri, nullptr, scratch_norm, nullptr, 0);
   const size_t stride = (size_t)ntri * nphi * nphi;
-  real_space_kernel<false><<<8 * ntri, 256, smem, s>>>(U, nb, N, nphi, E, 0, ntri, scratch_norm, nullptr,
-                                                       reinterpret_cast<double2*>(gamma), stride);
+  cudaError_t e = launch_real<kCounts>(ntri, smem, s, U, nb, N, nphi, E, 0, ntri, nullptr, scratch_norm, nullptr, 0);
+  if (e != cudaSuccess) return e;
+  e = launch_real<kGammaAdd>(8 * ntri, smem, s, U, nb, N, nphi, E, 0, ntri, scratch_norm, nullptr,
+                             reinterpret_cast<double2*>(gamma), stride);
+  if (e != cudaSuccess) return e;
   add_arrays<<<1024, 256, 0, s>>>(norm, scratch_norm, stride);
   return cudaGetLastError();
 }
@@ -266,11 +399,26 @@ size_t real_space_smem(int N, int nphi) {
   return (size_t)(nn * nn + nn * nphi) * sizeof(double2);
 }
 
+// bytes of scratch next to the Gamma chunk: e^{i phi} per bin and the exponential tables of a chunk
+size_t map4_table_bytes(int chunk_tri, int nphi, int n_ap) {
+  return (size_t)nphi * sizeof(double2) + (size_t)chunk_tri * 3 * nphi * n_ap * sizeof(double);
+}
+
+// Radial triples of one chunk: 256 MB of Gamma and tables, and whole rounds of two blocks per SM of
+// real_space_kernel (8 blocks a triple) where that leaves at least one.
+int map4_chunk(int ntri, int nphi, int n_ap) {
+  const size_t per = (size_t)nphi * nphi * 8 * sizeof(double2) + (size_t)3 * nphi * n_ap * sizeof(double);
+  const size_t fit = std::max<size_t>(1, (size_t)(256u << 20) / per);
+  if (fit >= (size_t)ntri) return ntri;
+  constexpr int kRound = 2 * 152 / 8;
+  return fit < kRound ? (int)fit : (int)(fit / kRound * kRound);
+}
+
 // Aperture measures: triples processed in chunks; returns per-(triple, slice, aperture)
 // partial sums in `partial` [ntri][nsplit][n_ap][8] complex, the angular bins of each
-// triple split into nsplit slices.
+// triple split into nsplit slices: 8 as the real-space blocks of the triple, more for a small chunk.
 int map4_nsplit(int chunk_tri, int ntri, int n_ap) {
-  int ns = (4 * 152 + chunk_tri - 1) / chunk_tri;
+  int ns = std::max(8, (4 * 152 + chunk_tri - 1) / chunk_tri);
   const size_t cap = (size_t)(256u << 20) / ((size_t)ntri * n_ap * 8 * 16);
   if ((size_t)ns > cap) ns = (int)cap;
   return ns < 1 ? 1 : (ns > 16 ? 16 : ns);
@@ -278,15 +426,17 @@ int map4_nsplit(int chunk_tri, int ntri, int n_ap) {
 
 cudaError_t map4_partials(const double* ups, const double* edges_host, int nb, int N, int nphi,
                           const double* ap_host, int n_ap, double* E_scratch, double* norm_chunk,
-                          double* gam_chunk, int chunk_tri, int nsplit, double* partial, cudaStream_t s) {
+                          double* gam_chunk, double* tables, int chunk_tri, int nsplit, double* partial,
+                          cudaStream_t s) {
   const int nn = 2 * N + 1;
   const int ntri = nb * nb * nb;
   angle_table<<<64, 256, 0, s>>>(N, nphi, reinterpret_cast<double2*>(E_scratch));
   ++g_launches;
   const size_t smem = (size_t)(nn * nn + nn * nphi) * sizeof(double2);
-  cudaError_t e = cudaFuncSetAttribute(real_space_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(real_space_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem4 = kM4Coef * kM4Row * sizeof(double2) + kM4Bins * (size_t)n_ap * sizeof(double);
+  // (the sums at the end, [parts][n_ap][kM4Coef] with parts n_ap <= 8 or parts = 1, fit in it)
+  static_assert(kM4Groups <= kM4Bins && 64 <= kM4Bins, "sums");
+  cudaError_t e = cudaFuncSetAttribute(map4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem4);
   if (e != cudaSuccess) return e;
   Map4Args a;
   a.nb = nb; a.nphi = nphi; a.n_ap = n_ap;
@@ -298,18 +448,24 @@ cudaError_t map4_partials(const double* ups, const double* edges_host, int nb, i
   for (int k = 0; k < n_ap; ++k) a.ap[k] = ap_host[k];
   const double2* U = reinterpret_cast<const double2*>(ups);
   const double2* E = reinterpret_cast<const double2*>(E_scratch);
+  double2* turn = reinterpret_cast<double2*>(tables);
+  double* tab = tables + 2 * (size_t)nphi;
+  double2* gam = reinterpret_cast<double2*>(gam_chunk);
   const size_t nph2 = (size_t)nphi * nphi;
+  map4_turns<<<(nphi + 127) / 128, 128, 0, s>>>(nphi, turn);
+  ++g_launches;
   for (int t0 = 0; t0 < ntri; t0 += chunk_tri) {
     const int nt = min(chunk_tri, ntri - t0);
     const size_t stride = (size_t)nt * nph2;
-    cudaMemsetAsync(gam_chunk, 0, 8 * stride * sizeof(double2), s);
-    real_space_kernel<true><<<nt, 256, smem, s>>>(U, nb, N, nphi, E, t0, nt, nullptr, norm_chunk, nullptr, 0);
-    real_space_kernel<false><<<8 * nt, 256, smem, s>>>(U, nb, N, nphi, E, t0, nt, norm_chunk, nullptr,
-                                                       reinterpret_cast<double2*>(gam_chunk), stride);
+    e = launch_real<kRecips>(nt, smem, s, U, nb, N, nphi, E, t0, nt, nullptr, norm_chunk, nullptr, 0);
+    if (e != cudaSuccess) return e;
+    e = launch_real<kGammaTimes>(8 * nt, smem, s, U, nb, N, nphi, E, t0, nt, norm_chunk, nullptr, gam, stride);
+    if (e != cudaSuccess) return e;
     a.tri0 = t0; a.ntri = nt;
-    map4_kernel<<<nt * nsplit, kM4Threads, 0, s>>>(a, reinterpret_cast<const double2*>(gam_chunk), stride,
-                                                   nsplit, reinterpret_cast<double2*>(partial));
-    g_launches += 3;
+    map4_tables<<<nt, 256, 0, s>>>(a, tab);
+    map4_kernel<<<nt * nsplit, kM4Threads, smem4, s>>>(a, gam, stride, tab, turn, nsplit,
+                                                       reinterpret_cast<double2*>(partial));
+    g_launches += 2;
   }
   return cudaGetLastError();
 }
@@ -318,17 +474,30 @@ namespace {
 
 // Sum the partials over triples and slices (fixed order), then the E/B split and the
 // Gaussian part.
-__global__ void map4_finish(const double2* __restrict__ partial, int nunits, int n_ap,
+constexpr int kM4FinThreads = 512;
+__global__ void __launch_bounds__(kM4FinThreads) map4_finish(const double2* __restrict__ partial, int nunits, int n_ap,
                             const double* __restrict__ xipm, const double* __restrict__ tb,
                             const double* __restrict__ area, int nb, const double* __restrict__ ap,
                             double* __restrict__ m4, double* __restrict__ eb, double* __restrict__ disc) {
   const int ia = blockIdx.x;
   __shared__ double2 mm[8];
   __shared__ double2 D[16];
+  __shared__ double2 run[kM4FinThreads];
+  {  // thread (stretch of the units, component), then the stretches in order
+    const int mu = threadIdx.x % 8, st = threadIdx.x / 8, ns = kM4FinThreads / 8;
+    const int u0 = (int)((long long)nunits * st / ns), u1 = (int)((long long)nunits * (st + 1) / ns);
+    double re = 0, im = 0;
+    for (int t = u0; t < u1; ++t) {
+      const double2 v = partial[((size_t)t * n_ap + ia) * 8 + mu];
+      re += v.x; im += v.y;
+    }
+    run[threadIdx.x] = make_double2(re, im);
+  }
+  __syncthreads();
   if (threadIdx.x < 8) {
     double re = 0, im = 0;
-    for (int t = 0; t < nunits; ++t) {
-      const double2 v = partial[((size_t)t * n_ap + ia) * 8 + threadIdx.x];
+    for (int st = 0; st < kM4FinThreads / 8; ++st) {
+      const double2 v = run[8 * st + threadIdx.x];
       re += v.x; im += v.y;
     }
     mm[threadIdx.x] = make_double2(re, im);
@@ -422,7 +591,7 @@ __global__ void map4_finish(const double2* __restrict__ partial, int nunits, int
 cudaError_t map4_finish_launch(const double* partial, int ntri, int n_ap, const double* d_xipm,
                                const double* d_tb, const double* d_area, int nb, const double* d_ap,
                                double* d_m4, double* d_eb, double* d_disc, cudaStream_t s) {
-  map4_finish<<<n_ap, 32, 0, s>>>(reinterpret_cast<const double2*>(partial), ntri, n_ap, d_xipm, d_tb,
+  map4_finish<<<n_ap, kM4FinThreads, 0, s>>>(reinterpret_cast<const double2*>(partial), ntri, n_ap, d_xipm, d_tb,
                                   d_area, nb, d_ap, d_m4, d_eb, d_disc);
   ++g_launches;
   return cudaGetLastError();
