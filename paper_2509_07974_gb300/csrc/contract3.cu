@@ -5,8 +5,8 @@
 // F_l = G_m, conj(G_m) or W_m with m = a n + b, and D the product of the two factors' terms of
 // one and the same neighbour (their sum over the bin is XX, XA or WW of the record), which
 // removes the triplets whose two neighbours coincide.  Records in FP64 or FP32, products and
-// sums in FP64.  One thread per (component, n, Theta1, Theta2, slice of the wave's centres),
-// each slice's centres summed in order; the slices' partial sums are then added in slice order.
+// sums in FP64, each slice's centres summed in order; the slices' partial sums are then added in
+// slice order.
 #include <algorithm>
 #include <cstdlib>
 
@@ -28,8 +28,14 @@ struct C3 {
   F3 f[2];
   D3 d;
 };
+// Component mu at n with (Theta1, Theta2) is component mir at -n with (Theta2, Theta1) where their
+// factors are each other's, swapped (mu 0, 1 and the normalisation with themselves, 2 with 3): of
+// such a pair only n >= 0, or only one component, is summed.  D does not depend on n.
 struct Table3 {
-  C3 c[5];  // mu = 0..3, 4: normalisation
+  C3 c[5];      // mu = 0..3, 4: normalisation
+  int mir[5];   // -1: none
+  int nitem;    // what is summed at |n|: component, sign of n (0 at n = 0 only once)
+  signed char mu[10], sg[10];
 };
 
 __device__ __forceinline__ double2 cj(double2 v) { return make_double2(v.x, -v.y); }
@@ -54,46 +60,104 @@ __device__ __forceinline__ double2 same_galaxy(const Cx* __restrict__ r, const L
   return d.conj ? cj(v) : v;
 }
 
-// block = (component and n, slice of the centres); thread = (Theta1, Theta2)
+// Block = (n >= 0, slice of the centres, 512 of the sums at +-n): the products of a sum are those of
+// two rows of nb factors, so kC3Centres centres at a time have their rows t F1 and F2 put into shared
+// memory as doubles and every sum takes one product from them.  The FP64 pipe bounds it (2
+// multiply-adds per clock and SM): four per sum and centre, where forming F1 F2, t and the same
+// neighbour's term for each sum took twelve, and all sums of |n| in one block leave few lanes idle.
+// 50000 centres, n_max = 20, 10 bins, FP32 records: 62 -> 7.3 ms.
+constexpr int kC3Threads = 256, kC3Out = 2, kC3Centres = 8;
 template <typename Cx>
-__global__ void contract3_kernel(const Layout L, const Table3 tab, const Cx* __restrict__ rec,
-                                 const Cx* __restrict__ xw, int T, int S, double2* __restrict__ part) {
-  const int nn = 2 * L.N + 1, nb = L.nb;
-  const int comp = blockIdx.x / S, sl = blockIdx.x % S;
-  const int mu = comp / nn, n = comp % nn - L.N;
-  const C3 c = tab.c[mu];
+__global__ void __launch_bounds__(kC3Threads) contract3_kernel(const Layout L, const Table3 tab,
+                                                               const Cx* __restrict__ rec,
+                                                               const Cx* __restrict__ xw, int T, int S, int chunks,
+                                                               double2* __restrict__ part) {
+  extern __shared__ double2 rows[];  // [kC3Centres][items of the block][2][nb]
+  const int nn = 2 * L.N + 1, nb = L.nb, nb2 = nb * nb, tid = threadIdx.x;
+  const int n = blockIdx.x / (S * chunks), sl = blockIdx.x / chunks % S, ch = blockIdx.x % chunks;
   const int i0 = (int)((long long)T * sl / S), i1 = (int)((long long)T * (sl + 1) / S);
-  for (int p = threadIdx.x; p < nb * nb; p += blockDim.x) {
-    const int b1 = p / nb, b2 = p % nb;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int i = i0; i < i1; ++i) {
-      const Cx* r = rec + (size_t)i * L.rec;
-      const double2 x = d2(xw[2 * (size_t)i]);
-      const double2 t = c.centre == 2 ? d2(xw[2 * (size_t)i + 1]) : (c.centre == 1 ? cj(x) : x);
-      double2 v = cmul(factor(r, L, c.f[0], n, b1), factor(r, L, c.f[1], n, b2));
-      if (b1 == b2) {
-        const double2 d = same_galaxy(r, L, c.d, b1);
-        v.x -= d.x;
-        v.y -= d.y;
+  const int o0 = ch * kC3Threads * kC3Out, o1 = min(o0 + kC3Threads * kC3Out, tab.nitem * nb2);
+  const int it0 = o0 / nb2, nit = (o1 - 1) / nb2 + 1 - it0, per = nit * 2 * nb;
+  int ra[kC3Out], rb[kC3Out];
+  double2 acc[kC3Out];
+#pragma unroll
+  for (int r = 0; r < kC3Out; ++r) {
+    const int o = o0 + r * kC3Threads + tid, it = o / nb2 - it0, b = o % nb2;
+    ra[r] = o < o1 ? it * 2 * nb + b / nb : -1;
+    rb[r] = it * 2 * nb + nb + b % nb;
+    acc[r] = make_double2(0.0, 0.0);
+  }
+  for (int i = i0; i < i1; i += kC3Centres) {
+    const int nc = min(kC3Centres, i1 - i);
+    __syncthreads();  // the rows before have been used
+    for (int k = tid; k < nc * per; k += kC3Threads) {
+      const int ci = i + k / per, e = k % per, it = it0 + e / (2 * nb), side = e / nb % 2, b = e % nb;
+      const C3& c = tab.c[tab.mu[it]];
+      double2 v = factor(rec + (size_t)ci * L.rec, L, c.f[side], tab.sg[it] * n, b);
+      if (side == 0) {
+        const double2 x = d2(xw[2 * (size_t)ci + (c.centre == 2)]);
+        v = cmul(c.centre == 1 ? cj(x) : x, v);
       }
-      acc = cadd(acc, cmul(t, v));
+      rows[k] = v;
     }
-    part[((size_t)sl * 5 * nn + comp) * nb * nb + p] = acc;
+    __syncthreads();
+    for (int k = 0; k < nc; ++k) {
+      const double2* rw = rows + k * per;
+#pragma unroll
+      for (int r = 0; r < kC3Out; ++r) {
+        if (ra[r] < 0) break;
+        const double2 u = rw[ra[r]], v = rw[rb[r]];
+        acc[r].x += u.x * v.x;
+        acc[r].y += u.x * v.y;
+        acc[r].x -= u.y * v.y;
+        acc[r].y += u.y * v.x;
+      }
+    }
+  }
+  double2* out = part + (size_t)sl * (5 * nn * nb2 + 5 * nb);
+#pragma unroll
+  for (int r = 0; r < kC3Out; ++r) {
+    if (ra[r] < 0) break;
+    const int o = o0 + r * kC3Threads + tid, it = o / nb2;
+    if (n == 0 && tab.sg[it] < 0) continue;  // the same sum as at + n
+    out[(size_t)(tab.mu[it] * nn + tab.sg[it] * n + L.N) * nb2 + o % nb2] = acc[r];
+  }
+  // the same neighbour's terms t D of the slice
+  if (n == 0 && ch == 0) {
+    for (int k = tid; k < 5 * nb; k += kC3Threads) {
+      const C3& c = tab.c[k / nb];
+      double2 sum = make_double2(0.0, 0.0);
+#pragma unroll 4
+      for (int i = i0; i < i1; ++i) {
+        const double2 x = d2(xw[2 * (size_t)i + (c.centre == 2)]);
+        sum = cadd(sum, cmul(c.centre == 1 ? cj(x) : x, same_galaxy(rec + (size_t)i * L.rec, L, c.d, k % nb)));
+      }
+      out[(size_t)5 * nn * nb2 + k] = sum;
+    }
   }
 }
 
 // thread = output entry: the slices' partial sums in slice order, with the component's sign
 __global__ void contract3_sum(const Layout L, const Table3 tab, int S, const double2* __restrict__ part,
                               double* __restrict__ ups3) {
-  const int nn = 2 * L.N + 1, nb2 = L.nb * L.nb;
-  const size_t total = (size_t)5 * nn * nb2;
+  const int nn = 2 * L.N + 1, nb = L.nb, nb2 = nb * nb;
+  const size_t total = (size_t)5 * nn * nb2, stride = total + 5 * nb;
   for (size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (size_t)gridDim.x * blockDim.x) {
-    const int mu = (int)(o / ((size_t)nn * nb2));
+    const int mu = (int)(o / ((size_t)nn * nb2)), n = (int)(o / nb2 % nn) - L.N;
+    const int b1 = (int)(o % nb2) / nb, b2 = (int)(o % nb2) % nb;
+    const int m = tab.mir[mu];
+    const bool mirrored = m >= 0 && (m == mu ? n < 0 : m > mu);
+    const size_t src = mirrored ? (size_t)(m * nn - n + L.N) * nb2 + b2 * nb + b1 : o;
     double re = 0.0, im = 0.0;
     for (int sl = 0; sl < S; ++sl) {
-      const double2 v = part[(size_t)sl * total + o];
+      const double2 v = part[(size_t)sl * stride + src];
       re += v.x;
       im += v.y;
+      if (b1 == b2) {
+        const double2 d = part[(size_t)sl * stride + total + mu * nb + b1];
+        re -= d.x;
+        im -= d.y;
+      }
     }
     ups3[2 * o] += tab.c[mu].sign * re;
     ups3[2 * o + 1] += tab.c[mu].sign * im;
@@ -142,6 +206,20 @@ bool build_table3(int N, Table3& t) {
     }
     if (!in_range(f0, N, -2 * N - 3, 2 * N - 1) || !in_range(f1, N, -2 * N - 3, 2 * N - 1)) return false;
   }
+  auto same = [](const F3& f, const F3& g) { return f.arr == g.arr && f.conj == g.conj && f.a == -g.a && f.b == g.b; };
+  t.nitem = 0;
+  for (int k = 0; k < 5; ++k) {
+    t.mir[k] = -1;
+    for (int m = 0; m < 5 && t.mir[k] < 0; ++m)
+      if (t.c[m].centre == t.c[k].centre && same(t.c[m].f[0], t.c[k].f[1]) && same(t.c[m].f[1], t.c[k].f[0]))
+        t.mir[k] = m;
+    if (t.mir[k] > k) continue;  // taken from that component
+    for (int sg = 1; sg >= -1; sg -= 2)
+      if (sg > 0 || t.mir[k] != k) {
+        t.mu[t.nitem] = (signed char)k;
+        t.sg[t.nitem++] = (signed char)sg;
+      }
+  }
   return true;
 }
 
@@ -152,9 +230,10 @@ bool contract3_supported(int N) {
   return build_table3(N, t);
 }
 
-int contract3_slices(int T) { return std::max(1, std::min(32, T / 128)); }
+// at least 32 centres to a slice
+int contract3_slices(int T) { return std::max(1, std::min(32, T / 32)); }
 size_t contract3_scratch_bytes(const Layout& L, int T) {
-  return (size_t)contract3_slices(T) * 5 * (2 * L.N + 1) * L.nb * L.nb * sizeof(double2);
+  return (size_t)contract3_slices(T) * 5 * ((2 * L.N + 1) * L.nb * L.nb + L.nb) * sizeof(double2);
 }
 
 template <typename Cx>
@@ -164,8 +243,15 @@ cudaError_t contract3_wave(const Layout& L, const Cx* rec, const Cx* xw, int T, 
   if (!build_table3(L.N, t)) return cudaErrorInvalidValue;
   if (T <= 0) return cudaSuccess;
   const int S = contract3_slices(T);
-  contract3_kernel<Cx><<<5 * (2 * L.N + 1) * S, 128, 0, s>>>(L, t, rec, xw, T, S, scratch);
-  contract3_sum<<<64, 256, 0, s>>>(L, t, S, scratch, ups3);
+  const int nb2 = L.nb * L.nb, outs = kC3Threads * kC3Out, chunks = (t.nitem * nb2 + outs - 1) / outs;
+  // components that 512 consecutive sums touch, at most
+  const int items = std::min(t.nitem, (outs + nb2 - 2) / nb2 + 1);
+  const size_t smem = (size_t)kC3Centres * items * 2 * L.nb * sizeof(double2);
+  cudaError_t e = cudaFuncSetAttribute(contract3_kernel<Cx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  contract3_kernel<Cx><<<(L.N + 1) * S * chunks, kC3Threads, smem, s>>>(L, t, rec, xw, T, S, chunks, scratch);
+  const int total = 5 * (2 * L.N + 1) * nb2;
+  contract3_sum<<<std::min(4 * 152, (total + 127) / 128), 128, 0, s>>>(L, t, S, scratch, ups3);
   g_launches += 2;
   return cudaGetLastError();
 }
