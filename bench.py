@@ -79,6 +79,10 @@ def gather_flop_per_pair(nmax):
     return 8 * (4 * N + 3) + 8 * (4 * N + 5) + 4 * ((2 * N + 1) + (2 * N + 3) + (2 * N + 1)) + 6 * (2 * N + 6) + 40
 
 
+GATHER_NOTE = ("the sums taken power by power; dense catalogues are summed through angular sectors (csrc/gather_sector.cu), "
+               "which executes about a fifth of these operations, so frac is not the FMA pipe's use")
+
+
 def contraction_flop(n_centres, nmax, nb):
     """One complex multiply-add per output element per centre: 8 * centres * 9 (2N+1)^2 nb^3."""
     return 8.0 * n_centres * 9 * (2 * nmax + 1) ** 2 * nb ** 3
@@ -541,11 +545,10 @@ def run_ours(args):
               "frac": g_ach / fp32_peak, "traffic": None, "ms_per_launch": g_ms,
               "peak_note": "FP32 FMA pipe: 152 SMs x 128 lanes x 2 FLOP x max SM clock (%s MHz)"
                            % pk.get("sm_max_mhz", 2070.0),
-              "algorithmic_flop_per_pair": flop_pair}
+              "algorithmic_flop_per_pair": flop_pair, "algorithmic_note": GATHER_NOTE}
     roof_c = {"bound": "tensor", "kernel": "contraction", "achieved": contraction_tflops, "peak": tf32_peak,
               "unit": "TFLOP/s", "frac": (contraction_tflops or 0.0) / tf32_peak, "traffic": None,
               "ms_per_launch": c_ms,
-              "frac_issued": (contraction_tflops or 0.0) * passes / tf32_peak,
               "passes": passes,
               "peak_note": ("kind::f16 dense: measured sustained bf16 (%s TFLOP/s, %s)"
                             % (pk.get("bf16_tflops_sustained"), pk.get("source"))) if f16_kind else
@@ -553,14 +556,15 @@ def run_ours(args):
                             "(not a measured tf32 rate)" % (pk.get("bf16_tflops_sustained"), pk.get("source"))),
               "algorithmic_flop_per_centre": c_flop / max(1, bd["centres"]),
               "algorithmic_note": ("complex multiply-adds of the symmetry-reduced contraction (bin pairs "
-                                   "Theta2 <= Theta3); all ordered triples would be %.4g FLOP per centre, "
+                                   "Theta2 <= Theta3), of which the f16x3 form executes the sums independent "
+                                   "under all exchanges of bins only; all ordered triples would be %.4g FLOP per centre, "
                                    "%.3g TFLOP/s equivalent" % (c_flop_full / max(1, bd["centres"]),
                                    c_flop_full / (bd["ms_contract"] / 1e3) / 1e12 if bd["ms_contract"] > 0 else 0.0))
                                   if tc_form else "complex multiply-adds of all ordered bin triples"}
     # DRAM bytes (read + write) of one full-size launch of the default configuration, from the
     # committed ncu summaries (null when the kernel source changed since the capture)
     if args.n_gal is None and args.centres is None:
-        roof_g["traffic"] = measured_traffic("gather_kernel")
+        roof_g["traffic"] = measured_traffic("gather_sector_kernel")
         roof_c["traffic"] = measured_traffic("contract_h16_kernel" if args.precision == "f16x3"
                                              else "contract_tc_kernel" if tc_form else "contract_kernel")
         roof_g["traffic_unit"] = roof_c["traffic_unit"] = "bytes per launch (DRAM read + write, ncu)"
@@ -807,9 +811,9 @@ def run_batched(args, kind):
     roof_g = {"bound": "alu", "kernel": "gather", "achieved": g_ach, "peak": fp32_peak, "unit": "TFLOP/s",
               "frac": g_ach / fp32_peak, "traffic": None, "ms_per_launch": g_ms,
               "peak_note": "FP32 FMA pipe: 152 SMs x 128 lanes x 2 FLOP x max SM clock",
-              "algorithmic_flop_per_pair": flop_pair}
+              "algorithmic_flop_per_pair": flop_pair, "algorithmic_note": GATHER_NOTE}
     roof_c = {"bound": "tensor", "kernel": "contraction", "achieved": c_tflops, "peak": peak_c, "unit": "TFLOP/s",
-              "frac": (c_tflops or 0.0) / peak_c, "frac_issued": 3 * (c_tflops or 0.0) / peak_c, "passes": 3,
+              "frac": (c_tflops or 0.0) / peak_c, "passes": 3,
               "traffic": None, "ms_per_launch": bd["ms_contract"] / waves,
               "peak_note": "kind::f16 dense: measured sustained bf16 (%s TFLOP/s, %s)"
                            % (pk.get("bf16_tflops_sustained"), pk.get("source")),

@@ -234,6 +234,11 @@ cudaError_t reduce_batch(const double* pos, const double* shear, const double* w
 cudaError_t gather_wave32(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
                           const WavePlan& plan, bool accumulate, float2* rec, float2* xw,
                           unsigned long long* pair_count, cudaStream_t s);
+// gather_sector.cu: the centres of dense catalogues, mb powers to each of nblk blocks; *dense_min: the
+// mean number of candidates from which on it takes a catalogue (0: none)
+cudaError_t gather_sector(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
+                          const WavePlan& plan, bool accumulate, int mb, int nblk, float2* rec, float2* xw,
+                          unsigned long long* pair_count, cudaStream_t s, float* dense_min);
 cudaError_t gather_wave64(const SortedCat& cat, const SortedCat& cen, const Bins& bins, const Layout& L,
                           const WavePlan& plan, bool accumulate, double2* rec, double2* xw,
                           unsigned long long* pair_count, cudaStream_t s);

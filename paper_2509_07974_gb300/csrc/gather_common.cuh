@@ -66,13 +66,9 @@ template <> struct Pair<double> {
 };
 
 template <> struct Pair<float> {
-  __device__ static int classify(const SortedCat& cat, int q, double cx, double cy, const float4& P,
-                                 const double* e2, const float* e2f, const float* win, const BinLookup& lk,
-                                 int nb, float& ur, float& ui) {
-    float4 Q = cat.p4[q];
-    float dx = (Q.x - P.x) + (Q.z - P.z);
-    float dy = (Q.y - P.y) + (Q.w - P.w);
-    float r2 = dx * dx + dy * dy;
+  // the bin of candidate q at the offset (dx, dy), r2 = dx^2 + dy^2 (or -1)
+  __device__ static int bin(const SortedCat& cat, int q, double cx, double cy, float r2, const double* e2,
+                            const float* e2f, const float* win, const BinLookup& lk, int nb) {
     int b;
     // the float decision stands unless r2 is within the edge's rounding window
     if (r2 < lk.out_lo || r2 >= lk.out_hi) return -1;
@@ -89,6 +85,16 @@ template <> struct Pair<float> {
     else if (b == nb) near = true;
     else near = (r2 - e2f[b] < win[b]) || (e2f[b + 1] - r2 <= win[b + 1]);
     if (near) b = classify_f64(cat.px[q] - cx, cat.py[q] - cy, e2, nb);
+    return b;
+  }
+  __device__ static int classify(const SortedCat& cat, int q, double cx, double cy, const float4& P,
+                                 const double* e2, const float* e2f, const float* win, const BinLookup& lk,
+                                 int nb, float& ur, float& ui) {
+    float4 Q = cat.p4[q];
+    float dx = (Q.x - P.x) + (Q.z - P.z);
+    float dy = (Q.y - P.y) + (Q.w - P.w);
+    float r2 = dx * dx + dy * dy;
+    const int b = bin(cat, q, cx, cy, r2, e2, e2f, win, lk, nb);
     if (b >= 0) {
       float rinv = rsqrtf(r2);
       ur = dx * rinv; ui = dy * rinv;
@@ -122,7 +128,16 @@ struct GatherArgs {
   int mb;    // powers per warp block (<= MB)
   int nblk;  // power blocks
   unsigned long long* pair_count;
+  float dense_min;  // FP32: centres of catalogues at least this dense go to gather_sector (0: none)
 };
+
+// Neighbours a centre of the segment finds on average (its catalogue over its grid's area).
+__device__ __forceinline__ float mean_candidates(const WaveSeg& sg, float rmax) {
+  const GridGeom& g = *sg.geom;
+  const int nc = g.ncx * g.ncy;
+  const float n = (float)(sg.cell_start[nc] - sg.cell_start[0]), q = rmax / g.cellf;
+  return n * fminf(1.f, 3.14159265f * q * q / (float)nc);
+}
 
 }  // namespace
 }  // namespace ext4pcf

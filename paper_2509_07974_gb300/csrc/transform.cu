@@ -370,7 +370,8 @@ cudaError_t launch_real(int blocks, size_t smem, cudaStream_t s, const double2* 
                         size_t stride) {
   cudaError_t e = cudaFuncSetAttribute(real_space_kernel<OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  real_space_kernel<OUT><<<blocks, kRealThreads, smem, s>>>(U, nb, N, nphi, E, tri0, ntri, norm_in, norm_out, gam, stride);
+  real_space_kernel<OUT><<<blocks, kRealThreads, smem, s>>>(U, nb, N, nphi, E, tri0, ntri, norm_in, norm_out, gam,
+                                                            stride);
   ++g_launches;
   return cudaGetLastError();
 }
