@@ -21,8 +21,8 @@
 //                    in FP32 and accumulates the eight power sums of a and w, in FP32 over at
 //                    most 32 galaxies per lane and then into unevaluated FP32 pairs (hi + lo,
 //                    error-free two-sum), reduced across the warp the same way;
-//   aperture_finish  one thread per aperture: adds the splits in order in FP64, applies
-//                    Newton's identities and writes the aperture record; one partial sum of
+//   aperture_finish  one thread per aperture, eight where there are many splits: adds the splits
+//                    in a fixed order in FP64, applies Newton's identities and writes the aperture record; one partial sum of
 //                    the records per block;
 //   aperture_moments one CTA: adds the block partials in order into the per-radius sums and
 //                    derives <M_ap^4>, <M_ap^2> and the connected part.
@@ -232,16 +232,22 @@ __device__ __forceinline__ void newton(const double p[5], double n, double& e1, 
 
 constexpr int kFinThreads = 128;
 
+// Threads to an aperture: few large apertures have many splits (up to some hundred), whose loads one
+// thread waits for one after another (30 us a radius, 17 us with eight).  The line is where eight
+// threads have a split each.
+int fin_group(int nsplit) { return nsplit >= 8 ? 8 : 1; }
+
+template <int G>
 __global__ void __launch_bounds__(kFinThreads) aperture_finish(const float* __restrict__ sums, int n_ap, int nsplit,
                                                                double theta, double* __restrict__ rec,
                                                                double* __restrict__ part) {
   __shared__ double red[4][kFinThreads];
-  const int ap = blockIdx.x * kFinThreads + threadIdx.x;
+  const int ap = (int)(((long long)blockIdx.x * kFinThreads + threadIdx.x) / G), sub = threadIdx.x % G;
   double t[4] = {0, 0, 0, 0};
-  if (ap < n_ap) {
-    double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long n = 0;
-    for (int sp = 0; sp < nsplit; ++sp) {
+  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  long long n = 0;
+  if (ap < n_ap)
+    for (int sp = sub; sp < nsplit; sp += G) {
       const float4* q = reinterpret_cast<const float4*>(sums + ((long long)ap * nsplit + sp) * kSumFloats);
       for (int i = 0; i < 4; ++i) {
         const float4 v = q[i];
@@ -250,6 +256,12 @@ __global__ void __launch_bounds__(kFinThreads) aperture_finish(const float* __re
       }
       n += __float_as_int(q[4].x);
     }
+#pragma unroll
+  for (int o = 1; o < G; o <<= 1) {
+    for (int i = 0; i < 8; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+    n += __shfl_xor_sync(0xffffffffu, n, o);
+  }
+  if (ap < n_ap && sub == 0) {
     const double c = 1.0 / (4.0 * M_PI * theta * theta);  // a = b c
     const double pa[5] = {0.0, s[0] * c, s[1] * c * c, s[2] * c * c * c, s[3] * (c * c) * (c * c)};
     const double pw[5] = {0.0, s[4], s[5], s[6], s[7]};
@@ -309,13 +321,14 @@ int map_direct_splits(int n_ap, int sm_count, double theta, double cell) {
 }
 
 size_t map_direct_scratch(int n_ap, int nsplit) {
-  const size_t nblk = (size_t)(n_ap + kFinThreads - 1) / kFinThreads;
+  const size_t nblk = ((size_t)n_ap * fin_group(nsplit) + kFinThreads - 1) / kFinThreads;
   return (size_t)n_ap * 16 + (size_t)n_ap * nsplit * kSumFloats * 4 + nblk * 32 + 256;
 }
 
 cudaError_t map_direct_radius(const SortedCat& cat, const double* centres, int n_ap, double theta,
                               int nsplit, void* scratch, double* rec, double* mom, cudaStream_t s) {
-  const int nblk = (n_ap + kFinThreads - 1) / kFinThreads;
+  const int group = fin_group(nsplit);
+  const int nblk = (int)(((long long)n_ap * group + kFinThreads - 1) / kFinThreads);
   int4* prep = (int4*)scratch;
   float* sums = (float*)((char*)scratch + (size_t)n_ap * 16);
   double* part = (double*)((char*)sums + (((size_t)n_ap * nsplit * kSumFloats * 4 + 255) / 256) * 256);
@@ -339,7 +352,8 @@ cudaError_t map_direct_radius(const SortedCat& cat, const double* centres, int n
       cudaError_t e = cudaMemsetAsync(sums, 0, (size_t)n_items * kSumFloats * 4, s);
       if (e != cudaSuccess) return e;
     }
-    aperture_finish<<<nblk, kFinThreads, 0, s>>>(sums, n_ap, nsplit, theta, rec, part);
+    if (group == 8) aperture_finish<8><<<nblk, kFinThreads, 0, s>>>(sums, n_ap, nsplit, theta, rec, part);
+    else aperture_finish<1><<<nblk, kFinThreads, 0, s>>>(sums, n_ap, nsplit, theta, rec, part);
     ++g_launches;
   }
   aperture_moments<<<1, kMomThreads, 0, s>>>(part, nblk, n_ap, theta, mom);
