@@ -11,17 +11,17 @@
 // One CTA (12 warps of 168 registers, one CTA per SM: the moments take a third of its shared memory)
 // takes centres in turn:
 //   (a) rows of cells as in gather.cu (found by one warp while the others finish the centre before);
-//       3840 candidates at a time are classified, four groups of a warp at once, and bucketed by (bin,
+//       3840 candidates at a time are classified, five groups of a warp at once, and bucketed by (bin,
 //       sector) in a stable order, so the summation order is deterministic;
-//   (b) items (bin, some of its sectors): two or four lanes per sector walk its pairs, 7 K + 9 sums in
+//   (b) items (bin, eight of its sectors): four lanes per sector walk its pairs, 7 K + 9 sums in
 //       registers, which are then added to the bin's moments in shared memory.  At most four bins, the
 //       widest, have sectors; the pairs of the others, few, are set aside and summed power by power;
 //   (c) at the end the moments become the record's entries, in place.
-// Measured: 8192 centres with 28000 candidates each, n_max = 20, 11.1 -> 8.6 ms; 256 centres of four
-// patches, n_max = 30, three passes of the tree approximation, 7.6 -> 3.8 ms.  Sums in fewer and
-// shorter chains, so the error against 64 bits falls too (9 bins, n_max = 16, FP32 contraction: 5.4e-7 ->
-// 1.6e-7 of the result).  No unit is saturated: with three warps to a scheduler the latencies of (a)
-// and the unequal sectors of (b) are what is left, issue slots 0.5 used.
+// Measured: 8192 centres with 28000 candidates each, n_max = 20, 11.1 -> 8.0 ms; 256 centres of four
+// patches, n_max = 30, three passes of the tree approximation, 7.6 -> 3.6 ms.  The records' error
+// against 64 bits stays (7.1e-8 -> 6.9e-8 of the largest; 100000 galaxies, 7 bins, n_max = 15).  No
+// unit is saturated: with three warps to a scheduler the latencies of (a) and the unequal sectors of
+// (b) are what is left, issue slots half used.
 #include <algorithm>
 #include <cmath>
 
@@ -77,15 +77,14 @@ constexpr int kMomRows = 7 * K + 12;
 // column of sector c in row r of the moments: the rows that a warp adds to at once on different banks
 __device__ __forceinline__ int mom_col(int c, int r) { return (c + 16 * (r & 1) + 8 * (r >> 1 & 1)) & (kSec - 1); }
 
-// Moments of one (bin, 32 / P sectors): P lanes to a sector, each every P-th of its pairs.  U_k = T_k
+// Moments of one (bin, eight sectors): four lanes to a sector, each every fourth of its pairs.  U_k = T_k
 // (-1)^{k/2} obeys U_{k+1} = -+ 2 t U_k + U_{k-1} (no subtraction, which the packed multiply-add
 // lacks; the signs cancel those of i^k in the transform); both halves of a packed pair hold the same
 // U_k.  Also the triple sums, with e^{-4 i delta} from its series.
-template <int K, int P>
+template <int K>
 __device__ __forceinline__ void sector_item(const float4* __restrict__ pairs, const int* __restrict__ koff, int key0,
                                             int part, int lane, float* __restrict__ mom) {
-  constexpr int kPer = 32 / P;
-  const int sec = kPer * part + (lane & (kPer - 1)), sub = lane / kPer;
+  const int sec = 8 * part + (lane & 7), sub = lane >> 3;
   const int e1 = koff[key0 + sec + 1];
   float2 ax[K], aq[K], aw[K];
   float aww[K];
@@ -97,7 +96,7 @@ __device__ __forceinline__ void sector_item(const float4* __restrict__ pairs, co
   float tr[9];
 #pragma unroll
   for (int j = 0; j < 9; ++j) tr[j] = 0.f;
-  for (int e = koff[key0 + sec] + sub; e < e1; e += P) {
+  for (int e = koff[key0 + sec] + sub; e < e1; e += 4) {
     const float4 p = pairs[e];
     const float t = p.x, xr = p.y, xi = p.z, w = p.w;
     const float2 X = make_float2(xr, xi);
@@ -137,8 +136,8 @@ __device__ __forceinline__ void sector_item(const float4* __restrict__ pairs, co
     tr[8] += ww * w;
   }
   __syncwarp();
-  // the lanes of a sector: of rows 7 k + q the lower half of the warp takes the even ones, the upper
-  // half the odd ones; with four lanes the halves' halves again
+  // the four lanes of a sector: of the rows the lower half of the warp takes the even ones, the upper
+  // half the odd ones, and the halves' halves again
   float r[kMomRows<K>];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
@@ -154,21 +153,16 @@ __device__ __forceinline__ void sector_item(const float4* __restrict__ pairs, co
     const float keep = up ? r[j + 1] : r[j];
     r[j / 2] = keep + __shfl_xor_sync(kFull, send, 16);
   }
-  if (P == 2) {
+  const int up2 = lane >> 3 & 1;
 #pragma unroll
-    for (int j = 0; j < kMomRows<K> / 2; ++j) mom[(2 * j + up) * kSec + mom_col(sec, 2 * j + up)] += r[j];
-  } else {
-    const int up2 = lane >> 3 & 1;
-#pragma unroll
-    for (int j = 0; j < kMomRows<K> / 2; j += 2) {
-      const float send = up2 ? r[j] : r[j + 1];
-      const float keep = up2 ? r[j + 1] : r[j];
-      r[j / 2] = keep + __shfl_xor_sync(kFull, send, 8);
-    }
-    const int row = 2 * up2 + up;
-#pragma unroll
-    for (int j = 0; j < kMomRows<K> / 4; ++j) mom[(4 * j + row) * kSec + mom_col(sec, row)] += r[j];
+  for (int j = 0; j < kMomRows<K> / 2; j += 2) {
+    const float send = up2 ? r[j] : r[j + 1];
+    const float keep = up2 ? r[j + 1] : r[j];
+    r[j / 2] = keep + __shfl_xor_sync(kFull, send, 8);
   }
+  const int row = 2 * up2 + up;
+#pragma unroll
+  for (int j = 0; j < kMomRows<K> / 4; ++j) mom[(4 * j + row) * kSec + mom_col(sec, row)] += r[j];
 }
 
 template <int W, int OFF>
@@ -549,7 +543,7 @@ gather_sector_kernel(const __grid_constant__ SectorArgs args, float2* __restrict
       static_assert((kWarps * kKeys + 3 * kCap) * 4 <= kCap * (int)sizeof(float4), "the pairs' memory");
       for (int k = lane; k < nkeys; k += 32) same[k] = 0;
       __syncwarp();
-      constexpr int kB = 4;  // groups of a warp on their way at once
+      constexpr int kB = 5;  // groups of a warp on their way at once
 #pragma unroll 1
       for (int ga0 = g0; ga0 < g1; ga0 += kB) {
         float4 Qs[kB];
@@ -698,26 +692,17 @@ gather_sector_kernel(const __grid_constant__ SectorArgs args, float2* __restrict
       __syncthreads();
       for (int i = lane; i < nkeys; i += 32) wc[i] = 0;  // for the next round
       if (mode == 0) pairs_here += (unsigned long long)koff[nkeys];
-      // ---- items, each taken by the next free warp: quarters of the bins with sectors (eighths of one
-      // with more than two fifths of the pairs, or a few warps would have most of the work); (bin,
-      // power block) of the others
-      unsigned fine = 0;
-      if (mode == 0) {
-        const int k0 = 1 + kSec * (lane < nbig ? lane : 0);
-        fine = __ballot_sync(kFull, lane < nbig && 5 * (koff[k0 + kSec] - koff[k0]) > 2 * koff[nkeys]);
-      }
-      const int nitems = mode == 0 ? 4 * (nbig + __popc(fine)) : nsmall * nblk;
+      // ---- items, each taken by the next free warp: eight sectors of a bin (quarters of the bins took
+      // 7% more of the whole: fewer items, and lanes less evenly filled), (bin, power block) of the
+      // bins without
+      const int nitems = mode == 0 ? 8 * nbig : nsmall * nblk;
       for (int item = warp; item < nitems;) {
         int next = 0;  // asked for now, used at the end
         if (lane == 0) next = kWarps + atomicAdd(&misc[4], 1);
         if (mode == 0) {
-          int slot = 0, part = item;
-          for (int n; part >= (n = fine >> slot & 1 ? 8 : 4); ++slot) part -= n;
-          const int key0 = 1 + kSec * slot;
-          float* m = mom + (size_t)slot * kRows * kSec;
-          if (fine >> slot & 1) sector_item<K, 4>(pairs, koff, key0, part, lane, m);
-          else if (koff[key0 + 16 * part] < koff[key0 + 16 * part + 16])
-            sector_item<K, 2>(pairs, koff, key0, part, lane, m);
+          const int slot = item >> 3, part = item & 7, key0 = 1 + kSec * slot;
+          if (koff[key0 + 8 * part] < koff[key0 + 8 * part + 8])
+            sector_item<K>(pairs, koff, key0, part, lane, mom + (size_t)slot * kRows * kSec);
         } else {
           const int i = item / nblk, b = order[nbig + i], k = item % nblk;
           if (koff[i] < koff[i + 1])
