@@ -25,8 +25,6 @@
 // to ~1e-7 of the cell size; pairs whose r^2 lies within a few rounding errors of a bin edge are
 // re-decided from the double positions.  (gather64.cu: the FP64 form; gather_sector.cu: dense
 // catalogues, from where on is said there.)
-#include <algorithm>
-
 #include "common.cuh"
 #include "gather_common.cuh"
 
@@ -175,17 +173,14 @@ gather_kernel(const GatherArgs args, float2* __restrict__ rec, float2* __restric
   const SortedCat& cat = args.cat;
   const Layout L = args.L;
   const int nb = args.bins.nb, cap = args.cap, mb = args.mb, nblk = args.nblk;
-  // centres of dense catalogues are gather_sector's
-  auto dense = [&](int c) {
+  // Nothing for a block past a masked wave's centres, nor for one of a dense catalogue, which is
+  // gather_sector's.  (A block per centre all the same: the hardware's order balances them better than
+  // strides over fewer blocks, 7.6 against 7.8 ms for 24001 centres.)
+  {
     int j = 0;
-    const int si = seg_of(args.plan, c, &j);
-    return si >= 0 && j < seg_live(args.plan.seg[si]) &&
-           mean_candidates(args.plan.seg[si], (float)args.bins.rmax) >= args.dense_min;
-  };
-  if (args.dense_min > 0.f) {
-    int c = blockIdx.x;
-    while (c < args.plan.total && dense(c)) c += gridDim.x;
-    if (c >= args.plan.total) return;
+    const int si = seg_of(args.plan, blockIdx.x, &j);
+    if (si < 0 || j >= seg_live(args.plan.seg[si])) return;
+    if (args.dense_min > 0.f && mean_candidates(args.plan.seg[si], (float)args.bins.rmax) >= args.dense_min) return;
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -261,7 +256,6 @@ gather_kernel(const GatherArgs args, float2* __restrict__ rec, float2* __restric
     int j = 0;
     const int si = seg_of(args.plan, c, &j);
     if (si < 0 || j >= seg_live(args.plan.seg[si])) continue;  // uniform over the block
-    if (args.dense_min > 0.f && dense(c)) continue;
     const WaveSeg& sg = args.plan.seg[si];
     const GridGeom gm = *sg.geom;
     const double gx0 = gm.x0, gy0 = gm.y0, cell = gm.cell;
@@ -456,9 +450,7 @@ cudaError_t gather_wave32(const SortedCat& cat, const SortedCat& cen, const Bins
   a.dense_min = 0.f;
   e = gather_sector(cat, cen, bins, L, plan, accumulate, a.mb, a.nblk, rec, xw, pair_count, s, &a.dense_min);
   if (e != cudaSuccess) return e;
-  // with the dense centres gone few blocks do anything: as many as find a place at once, four times
-  const int blocks = a.dense_min > 0.f ? std::min(plan.total, 4 * 2 * 152) : plan.total;
-  gather_kernel<<<blocks, kThreads, smem, s>>>(a, rec, xw);
+  gather_kernel<<<plan.total, kThreads, smem, s>>>(a, rec, xw);
   ++g_launches;
   return cudaGetLastError();
 }
