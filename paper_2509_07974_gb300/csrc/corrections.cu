@@ -4,8 +4,9 @@
 // One block takes one sg and one slice of the wave's centres.  It stages the two merged factors XX_sg
 // and XA_{sg+4} and the four columns x G_{-sg-8}, x^* G_{-sg-4}, x G_{sg+4}^*, x^* G_sg^* of 32 centres
 // (each loaded once for the six arrays they serve), and a thread holds a 2 x 2 tile of bins of one
-// array.  Products and sums over 16 centres are in R, the rest in FP64; every slice adds into a copy
-// of its own (one writer, no atomics), and the copies are added in order at the end of the call.
+// array, or with few bins its part of the centres.  Products and sums over corr_run centres are in R,
+// the rest in FP64; every slice adds into a copy of its own (one writer, no atomics), and the copies
+// are added in order at the end of the call.
 // One block per (component, kind, index), 27 arrays of terms where seven hold them all, took 1.56 ms
 // a wave of 8192 centres at n_max = 20, 10 bins (and the xi sums 76 us); this takes 0.52 ms, a
 // quarter of it FP64 additions (16 clocks a warp instruction and SM).
@@ -18,7 +19,16 @@ namespace ext4pcf {
 namespace {
 
 constexpr int kCorrChunk = 32;  // centres staged at once
-constexpr int kCorrRun = 16;    // centres summed in R before they are added in FP64
+
+// Few bins have few tiles: up to kCorrParts threads share one, each with every parts-th centre.
+constexpr int kCorrParts = 8;
+// Centres that a thread sums in FP32 before it adds them in FP64.  Few bins are the cheaper ones and keep
+// more of their sums in FP64: no more than the 1, 3, 7, 11, 19 ... centres that 192 threads sharing the
+// tiles of 2, 4, 6, 8, 10 ... bins have of 128 each.  (16 for every number of bins lost what lies 2^-24 below the
+// largest of 16 terms.)  Whole split-FP16 calls on 3000 galaxies with 16 everywhere, with these runs and one
+// thread to a tile, and as it is: 0.72, 1.07, 0.78 ms (2 bins, n_max = 20); 0.57, 0.67, 0.61 ms (4, 10);
+// 1.03, 1.13, 1.09 ms (5, 20).
+__host__ __device__ constexpr int corr_run(int nb) { return nb <= 2 ? 1 : nb <= 4 ? 2 : nb <= 6 ? 6 : nb <= 8 ? 8 : 16; }
 
 template <typename Cx> struct __align__(16) Pair2 { Cx a, b; };
 
@@ -96,6 +106,7 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
   const int sg = wk ? job - C.nsig : -2 * N - 6 + job;  // (W blocks: the index c)
   const int width = (wk ? 2 : 6) * nbp;                 // staged values per centre
   const int tiles = (wk ? 1 : 6) * nt * nt;
+  const int run = sizeof(R) == 4 ? corr_run(nb) : 16;
   Cx* st = reinterpret_cast<Cx*>(smem_raw);  // [kCorrChunk][width]
   // the value this thread stages of every (blockDim / width)-th centre: its place in a record (-1: a
   // zero), its conjugation and its centre factor (0: none, 1: x, 2: x^*, 3: w)
@@ -125,9 +136,11 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
       }
     }
   }
+  const int parts = max(1, min(kCorrParts, (int)blockDim.x / tiles));
   for (int i0 = 0; i0 < tiles; i0 += blockDim.x) {
-    const int tile = i0 + tid, k = tile / (nt * nt), ta = 2 * ((tile / nt) % nt), tb = 2 * (tile % nt);
-    const bool active = tile < tiles && (wk || corr_valid(L, k, sg));
+    const int tile = parts > 1 ? tid % tiles : i0 + tid, part = parts > 1 ? tid / tiles : 0;
+    const int k = tile / (nt * nt), ta = 2 * ((tile / nt) % nt), tb = 2 * (tile % nt);
+    const bool active = tile < tiles && part < parts && (wk || corr_valid(L, k, sg));
     const int po = wk ? ta : kArrP[active ? k : 0] * nbp + ta, oo = wk ? nbp + tb : (2 + kArrO[active ? k : 0]) * nbp + tb;
     for (int si = 0; si < plan.nseg; ++si) {
       const WaveSeg& g = plan.seg[si];
@@ -159,12 +172,12 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
         }
         __syncthreads();
         if (active) {
-          for (int h = 0; h < nc; h += kCorrRun) {
+          for (int h = part; h < nc; h += run * parts) {
             Cx acc[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[i] = cmk<Cx>(R(0), R(0));
-            const int he = min(nc, h + kCorrRun);
-            for (int cc = h; cc < he; ++cc) {
+            const int he = min(nc, h + run * parts);
+            for (int cc = h; cc < he; cc += parts) {
               const Cx* row = st + cc * width;  // (po, oo and width are even: aligned pairs)
               const Pair2<Cx> p = *reinterpret_cast<const Pair2<Cx>*>(row + po);
               const Pair2<Cx> o = *reinterpret_cast<const Pair2<Cx>*>(row + oo);
@@ -181,18 +194,32 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
           }
         }
       }
-      if (active) {
-        double2* o = copy + (size_t)g.slot * slot_stride + (wk ? C.ow + (size_t)sg * nb2 : ((size_t)k * C.nsig + job) * nb2);
+      double2* out = copy + (size_t)g.slot * slot_stride;
+      auto add = [&](int tl, int i, double2 sum) {  // value i of tile tl
+        const int a = tl / (nt * nt), ba = 2 * ((tl / nt) % nt) + (i >> 1), bb = 2 * (tl % nt) + (i & 1);
+        if (ba >= nb || bb >= nb || !(wk || corr_valid(L, a, sg))) return;
+        double2* o = out + (wk ? C.ow + (size_t)sg * nb2 : ((size_t)a * C.nsig + job) * nb2) + ba * nb + bb;
+        const double2 v = *o;
+        *o = make_double2(v.x + sum.x, v.y + sum.y);
+      };
+      if (parts > 1) {  // the parts' sums in order (the staged values have been used)
+        double2* red = reinterpret_cast<double2*>(smem_raw);  // [parts][tiles][4]
+        __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int ba = ta + (i >> 1), bb = tb + (i & 1);
-          if (ba < nb && bb < nb) {
-            double2 v = o[ba * nb + bb];
-            v.x += a64[i][0];
-            v.y += a64[i][1];
-            o[ba * nb + bb] = v;
+        for (int i = 0; i < 4; ++i)
+          if (part < parts) red[tid * 4 + i] = make_double2(a64[i][0], a64[i][1]);
+        __syncthreads();
+        for (int e = tid; e < 4 * tiles; e += blockDim.x) {
+          double2 sum = red[e];
+          for (int p = 1; p < parts; ++p) {
+            sum.x += red[e + p * 4 * tiles].x;
+            sum.y += red[e + p * 4 * tiles].y;
           }
+          add(e / 4, e % 4, sum);
         }
+      } else if (active) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) add(tile, i, make_double2(a64[i][0], a64[i][1]));
       }
     }
   }
@@ -235,8 +262,9 @@ cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t
   if (plan.total <= 0 || plan.nseg <= 0) return cudaSuccess;
   const CorrLayout C = CorrLayout::make(L.N, L.nb);
   const int nt = (L.nb + 1) / 2;
-  const int threads = std::min(384, std::max(160, (6 * nt * nt + 31) / 32 * 32));
-  const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>), (size_t)threads * sizeof(double2));
+  // up to eight bins 192 threads: 8, 8, 3 and 2 to a tile of the six X arrays
+  const int threads = std::min(384, std::max(nt <= 4 ? 192 : 160, (6 * nt * nt + 31) / 32 * 32));
+  const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>), (size_t)threads * 4 * sizeof(double2));
   cudaError_t e = cudaFuncSetAttribute(corrections_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   corrections_kernel<R><<<dim3(C.nsig + 2 * L.N + 2, corrections_copies(n_out)), threads, smem, s>>>(
