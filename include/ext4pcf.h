@@ -137,7 +137,7 @@ EXT4PCF_API int ext4pcf_synchronize(ext4pcf_ctx* ctx);
  *   n_gal       total galaxies over all catalogues (>= 0)
  *   radial_bins host, double [n_bins+1], strictly increasing, radial_bins[0] > 0
  *   n_bins      1..32 (1..16 for the tensor-core precisions TF32, 3XTF32, SPLIT_BF16 and SPLIT_F16, whose
- *               B tile holds at most 64 columns, 4 per bin; larger n_bins return
+ *               tiles are laid out for no more; larger n_bins return
  *               EXT4PCF_E_UNSUPPORTED before any work);  n_max >= 0 (<= 40).  A centre's
  *               record, n_bins (14 n_max + 18) complex values, must also fit the gather's
  *               shared memory: every n_max up to n_bins = 16; at n_bins = 20, 24, 28, 32,
@@ -328,14 +328,17 @@ EXT4PCF_API int ext4pcf_measure3(ext4pcf_ctx* ctx, const double* positions, cons
                                  const double* weights, int64_t n_gal, const double* radial_bins,
                                  int n_bins, int n_max, double* upsilon3);
 
-/* The factor tables compiled into the 4PCF contraction kernels, for inspection, in the
- * layout of ext4pcf_nth_order_factors at order 4 (row mu = 0..7, row 8 the normalisation;
- * 17 ints per row).
- *   which  0: CUDA-core contraction (FP64 / FP32 forms), 1: tensor-core contraction,
- *          2: the exchange of Theta2 and Theta3 used by the tensor-core contraction (Table
+/* The factors of the 4PCF contraction kernels, for inspection, in the layout of
+ * ext4pcf_nth_order_factors at order 4 (row mu = 0..7, row 8 the normalisation; 17 ints per
+ * row).
+ *   which  0: the FP64, FP32 and SPLIT_F16 forms, which sum what no permutation of the bins
+ *          turns into one another: derived from the map by which those sums are expanded into
+ *          the components and from their columns; 1: the table compiled into the 3XTF32,
+ *          SPLIT_BF16 and TF32 contraction;
+ *          2: the exchange of Theta2 and Theta3 used by the contraction of which = 1 (Table
  *          tab:4PCFSymm): per component mu the pair (mu', o) with
  *          Upsilon_mu[n2, n3](Th1, Th2, Th3) = Upsilon_mu'[n3 + o, n2 - o](Th1, Th3, Th2),
- *          derived from the tensor-core factor table (18 ints)
+ *          derived from its factor table (18 ints)
  *   table  host, int [9][17] (which 0, 1) or [9][2] (which 2), or NULL to query the size;
  *   cap    ints available
  * Host only.  Returns 153 (18 for which = 2), or EXT4PCF_E_INVALID_ARG. */

@@ -19,18 +19,18 @@ bool basis_make(const Layout& L, Basis& B) {
   std::vector<int> lo(B.nsg, 1 << 20), up(B.nsg, -(1 << 20));
   for (int n2 = -N; n2 <= N; ++n2)
     for (int n3 = -N; n3 <= N; ++n3)
-      for (int f = 0; f < 2; ++f) {  // the three multipole indices of F0 / F2 and of F1 / F3
-        const int s = n2 + n3;
-        const int k[3] = {f ? s - 1 : s - 3, -n2 - 2, f ? -n3 - 1 : -n3 - 3};
-        const int total = f ? -4 : -8;
-        for (int i = 0; i < 3; ++i)  // any of them can stand in the column's place
+      for (int mu = 0; mu < 8; ++mu) {
+        const BasisTerm t = basis_term(mu, n2, n3);
+        for (int i = 0; i < 3; ++i) {
+          if (t.q >= 2 && i != t.place) continue;  // (F0, F1: any factor can stand in the column's place)
+          const int q = basis_total(t.q) - t.k[i] - B.sg0;
+          if (q < 0 || q >= B.nsg) return false;
           for (int j = 0; j < 3; ++j) {
             if (i == j) continue;
-            const int q = total - k[i] - B.sg0;
-            if (q < 0 || q >= B.nsg) return false;
-            lo[q] = std::min(lo[q], k[j]);
-            up[q] = std::max(up[q], k[j]);
+            lo[q] = std::min(lo[q], t.k[j]);
+            up[q] = std::max(up[q], t.k[j]);
           }
+        }
       }
   B.rx = 0;
   for (int q = 0; q < B.nsg; ++q) {
@@ -71,19 +71,12 @@ __global__ void __launch_bounds__(kExpandThreads) expand_kernel(const __grid_con
                                                                 double2* __restrict__ ups) {
   extern __shared__ double2 merged[];  // [3][nb][nb]: factors (1, 2), (1, 3), (2, 3); triple [nb]
   const int N = B.N, nb = B.nb, np = B.npairs, nn = 2 * N + 1, nb2 = nb * nb, nb3 = nb2 * nb;
-  const int mu = blockIdx.x / (nn * nn), n2 = (blockIdx.x / nn) % nn - N, n3 = blockIdx.x % nn - N, s = n2 + n3;
+  const int mu = blockIdx.x / (nn * nn), n2 = (blockIdx.x / nn) % nn - N, n3 = blockIdx.x % nn - N;
   const size_t stride = B.elems();
-  const bool odd = mu == 1 || (mu >= 5 && mu < 8);  // x^* at the centre: F1 or F3
-  const bool flip = mu == 8 && s < 0;               // FW[-sg, -a] = FW[sg, a]^*
-  // family, place of its column among the three factors, sg of that column (families F2, F3) and
-  // the multipole index of every factor
-  const int q = mu == 8 ? 4 : mu < 2 ? mu : odd ? 3 : 2;
-  const int place = mu == 3 || mu == 6 ? 1 : mu == 4 || mu == 7 ? 2 : 0;
-  int k[3];
-  k[0] = mu == 8 ? (flip ? -s : s) : odd ? s - 1 : s - 3;
-  k[1] = mu == 8 ? (flip ? n2 : -n2) : -n2 - 2;
-  k[2] = mu == 8 ? (flip ? n3 : -n3) : odd ? -n3 - 1 : -n3 - 3;
-  const int sgc = place == 0 ? (odd ? -s - 3 : -s - 5) : place == 1 ? (odd ? n2 - 2 : n2 - 6) : odd ? n3 - 3 : n3 - 5;
+  const BasisTerm term = basis_term(mu, n2, n3);
+  const int q = term.q, place = term.place, sgc = term.sg, total = basis_total(q);
+  const int(&k)[3] = term.k;
+  const bool flip = term.flip;
   const CorrLayout C = CorrLayout::make(N, nb);
   for (int i = threadIdx.x; i < 3 * nb2 + nb; i += kExpandThreads) {
     double2 v;
@@ -98,7 +91,7 @@ __global__ void __launch_bounds__(kExpandThreads) expand_kernel(const __grid_con
       } else if (q >= 2 && third == place) {  // both row factors merged: the third is the column
         at = (size_t)(q == 2 ? 2 : 4) * C.nsig * nb2 + (size_t)(sgc + 2 * N + 6) * nb2;
       } else {
-        at = (size_t)(q < 2 ? q : q == 2 ? 3 : 5) * C.nsig * nb2 + (size_t)(2 * N + 6 - c - (odd ? 4 : 8)) * nb2;
+        at = (size_t)(q < 2 ? q : q == 2 ? 3 : 5) * C.nsig * nb2 + (size_t)(2 * N + 6 + total - c) * nb2;
       }
       v = corr[at + (i - m * nb2)];
       if (q == 4 && c < 0) v.y = -v.y;
@@ -123,7 +116,7 @@ __global__ void __launch_bounds__(kExpandThreads) expand_kernel(const __grid_con
       order2(k0, c0, k1, c1);
       order2(k1, c1, k2, c2);
       order2(k0, c0, k1, c1);
-      sg = (q ? -4 : -8) - k0;
+      sg = total - k0;
     } else if (q == 4) {
       order2(k1, c1, k2, c2);
     } else {
@@ -183,6 +176,33 @@ __global__ void __launch_bounds__(kExpandThreads) expand_kernel(const __grid_con
 }
 
 }  // namespace
+
+// The factors of every component from basis_term and the families' columns, in the layout of
+// ext4pcf_nth_order_factors at order 4: sign, centre code, then per bin (array, conj, coefficient of n2,
+// coefficient of n3, constant).  Indices are linear in (n2, n3) (for N at s >= 0, and past it by flip).
+int contraction_table_cc(int* out) {
+  for (int mu = 0; mu < 9; ++mu) {
+    int* t = out + mu * 17;
+    int idx[3][3];  // factor, at (0, 0), (1, 0), (0, 1)
+    for (int e = 0; e < 3; ++e) {
+      const BasisTerm b = basis_term(mu, e == 1, e == 2);
+      t[0] = 1;
+      t[1] = b.q == 4 ? 2 : basis_centre_conj(b.q);
+      for (int l = 0; l < 3; ++l) {
+        const bool column = b.q < 4 && l == b.place;
+        idx[l][e] = column ? basis_col_index(b.q, b.sg) : b.k[l];
+        t[2 + 5 * l] = b.q == 4;
+        t[3 + 5 * l] = column && basis_col_conj(b.q);
+      }
+    }
+    for (int l = 0; l < 3; ++l) {
+      t[4 + 5 * l] = idx[l][1] - idx[l][0];
+      t[5 + 5 * l] = idx[l][2] - idx[l][0];
+      t[6 + 5 * l] = idx[l][0];
+    }
+  }
+  return 9 * 17;
+}
 
 cudaError_t basis_expand(const Basis& B, const double* red, int slices, const double* corr, double* ups,
                          cudaStream_t s) {

@@ -53,6 +53,30 @@ __host__ __device__ inline bool basis_centre_conj(int q) { return (q & 1) != 0; 
 // G index within the record
 __host__ __device__ inline bool basis_in_g(int N, int m) { return m >= -2 * N - 3 && m <= 2 * N - 1; }
 
+// Where component mu (0..7, 8: N) at (n2, n3) is found among the families (the table above): the expansion,
+// the rows of the reduced array and the table of ext4pcf_contraction_tables all follow from this.
+// k: the multipole index of the factor of bins 1, 2, 3 (of a column of F2, F3, which is conjugated, the one
+// that F0, F1 would have in its place); place: the column's factor, sg: its sums' (F0 and F1 have any
+// factor in the column's place); flip: N at s < 0, the conjugate of the sum with these indices.
+struct BasisTerm {
+  int q, place, sg, k[3];
+  bool flip;
+};
+__host__ __device__ inline int basis_total(int q) { return q == 4 ? 0 : basis_centre_conj(q) ? -4 : -8; }  // sum of the k
+__host__ __device__ inline BasisTerm basis_term(int mu, int n2, int n3) {
+  const int s = n2 + n3;
+  const bool odd = mu == 1 || (mu >= 5 && mu < 8);  // x^* at the centre: F1 or F3
+  BasisTerm t;
+  t.q = mu == 8 ? 4 : mu < 2 ? mu : odd ? 3 : 2;
+  t.place = mu == 3 || mu == 6 ? 1 : mu == 4 || mu == 7 ? 2 : 0;
+  t.flip = mu == 8 && s < 0;  // FW[-sg, -a] = FW[sg, a]^*
+  t.k[0] = mu == 8 ? (t.flip ? -s : s) : odd ? s - 1 : s - 3;
+  t.k[1] = mu == 8 ? (t.flip ? n2 : -n2) : -n2 - 2;
+  t.k[2] = mu == 8 ? (t.flip ? n3 : -n3) : odd ? -n3 - 1 : -n3 - 3;
+  t.sg = basis_total(t.q) - (t.place == 0 ? t.k[0] : t.place == 1 ? t.k[1] : t.k[2]);
+  return t;
+}
+
 bool basis_make(const Layout& L, Basis& B);
 
 // bin pair p -> (b2, b3), b2 <= b3, pairs in row-major order of (b2, b3)

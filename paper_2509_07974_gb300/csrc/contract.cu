@@ -11,31 +11,6 @@ namespace ext4pcf {
 
 namespace {
 
-// Which per-centre array a factor reads and how its index follows from (s, n2, n3).
-enum Arr { kG = 0, kW = 1, kXX = 2, kXA = 3, kWW = 4 };
-struct Factor {
-  signed char arr, sgn, off, conj;
-};
-struct Comp {
-  signed char xconj;  // 0: x_i, 1: x_i^*, 2: w_i
-  Factor A, B, C;     // A(Theta1; s), B(Theta2; n2), C(Theta3; n3)
-};
-
-// Upsilon_0..7 (x-projection) and N: xt * A[s] * B[n2] * C[n3].
-#define EXT4PCF_COMP_TABLE                                                          \
-  {                                                                               \
-    {0, {kG, 1, -3, 0}, {kG, -1, -2, 0}, {kG, -1, -3, 0}},                        \
-    {1, {kG, 1, -1, 0}, {kG, -1, -2, 0}, {kG, -1, -1, 0}},                        \
-    {0, {kG, -1, -1, 1}, {kG, -1, -2, 0}, {kG, -1, -3, 0}},                       \
-    {0, {kG, 1, -3, 0}, {kG, 1, -2, 1}, {kG, -1, -3, 0}},                         \
-    {0, {kG, 1, -3, 0}, {kG, -1, -2, 0}, {kG, 1, -1, 1}},                         \
-    {1, {kG, -1, -3, 1}, {kG, -1, -2, 0}, {kG, -1, -1, 0}},                       \
-    {1, {kG, 1, -1, 0}, {kG, 1, -2, 1}, {kG, -1, -1, 0}},                         \
-    {1, {kG, 1, -1, 0}, {kG, -1, -2, 0}, {kG, 1, -3, 1}},                         \
-    {2, {kW, 1, 0, 0}, {kW, -1, 0, 0}, {kW, -1, 0, 0}},                           \
-  }
-const Comp kCompHost[9] = EXT4PCF_COMP_TABLE;
-
 constexpr int kChunk = 32;  // centres staged per pass of the contraction kernel
 
 // One thread per row (sg, a, b2 <= b3) of the reduced array: it forms the row product
@@ -229,26 +204,6 @@ template cudaError_t contract_wave<float>(const Layout&, const Basis&, const flo
                                           int, double*, cudaStream_t);
 template cudaError_t contract_wave<double>(const Layout&, const Basis&, const double2*, const double2*, int,
                                            const int*, int, double*, cudaStream_t);
-// kComp in the layout of ext4pcf_nth_order_factors at order 4: sign, centre code, then per
-// bin (array, conj, coefficient of n2, coefficient of n3, constant); A reads s = n2 + n3.
-int contraction_table_cc(int* out) {
-  for (int mu = 0; mu < 9; ++mu) {
-    const Comp& c = kCompHost[mu];
-    int* t = out + mu * 17;
-    t[0] = 1;
-    t[1] = c.xconj;
-    const Factor f[3] = {c.A, c.B, c.C};
-    for (int l = 0; l < 3; ++l) {
-      int* r = t + 2 + 5 * l;
-      r[0] = f[l].arr == kW ? 1 : 0;
-      r[1] = f[l].conj;
-      r[2] = (l == 0 || l == 1) ? f[l].sgn : 0;
-      r[3] = (l == 0 || l == 2) ? f[l].sgn : 0;
-      r[4] = f[l].off;
-    }
-  }
-  return 9 * 17;
-}
 
 }  // namespace ext4pcf
 

@@ -1,5 +1,5 @@
 // Factor table of the Khatri-Rao form of the 4PCF multipoles (Eq. 4PCFMultipoles with the
-// natural components of Sec. 3.1), shared by the tensor-core contraction kernels.
+// natural components of Sec. 3.1) of the 3xTF32, BF16x3 and TF32 contraction.
 //
 // For fixed s = n2 + n3 every natural component factorises as
 //   Upsilon_mu[n2,n3](Th1,Th2,Th3) = sum_i A_i^mu[s](Th1) * xt_i B_i[n2](Th2) C_i[n3](Th3).

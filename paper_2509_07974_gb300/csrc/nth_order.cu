@@ -1,8 +1,8 @@
 // Natural components of the shear N-point function and their multipole factorisation
 // (paper App. F): the tables that a multipole estimator of order N contracts, generated
 // from the sign matrix beta instead of written by hand.  Host code only (no GPU, no
-// context); the 4PCF contraction kernels carry hand-written tables of the same form, which
-// ext4pcf_contraction_tables exposes for comparison.
+// context); the 4PCF contraction kernels have their factors by hand, which
+// ext4pcf_contraction_tables gives in the same form for comparison.
 //
 // Enumeration (App. F.1): p = 0, 1, ..., floor(N/2) conjugated shears; for each p the sets
 // of conjugated positions in lexicographic order (the rightmost position advances first);

@@ -244,9 +244,9 @@ def ext4pcf_nth_order_factors(order, mu):
 
 
 def ext4pcf_contraction_tables(which):
-    """The 4PCF contraction kernels' own factor tables (0 CUDA-core, 1 tensor-core), int32 [9][17];
-    which = 2: the Theta2 <-> Theta3 map of the reduced tensor-core contraction, int32 [9][2]
-    (mu', o per component)."""
+    """The factors of the 4PCF contraction kernels (0: FP64, FP32 and split-FP16, 1: 3xTF32, BF16x3 and
+    TF32), int32 [9][17]; which = 2: the Theta2 <-> Theta3 map of the latter, int32 [9][2] (mu', o per
+    component)."""
     import numpy as np
     lib = load()
     n = _host_table(lib.ext4pcf_contraction_tables(int(which), None, 0))
