@@ -344,6 +344,13 @@ EXT4PCF_API int ext4pcf_measure3(ext4pcf_ctx* ctx, const double* positions, cons
  * Host only.  Returns 153 (18 for which = 2), or EXT4PCF_E_INVALID_ARG. */
 EXT4PCF_API int ext4pcf_contraction_tables(int which, int* table, int cap);
 
+/* Centres of the context's last ext4pcf_measure, ext4pcf_measure_batch, ext4pcf_multipoles or
+ * ext4pcf_measure3 call (of those that ran kernels) whose neighbours were summed through angular sectors (the FP32 gather of
+ * dense catalogues), for inspection; with the tree approximation a centre counts once for each of
+ * its passes that was.  Synchronises the context's stream.  Returns EXT4PCF_OK,
+ * EXT4PCF_E_INVALID_ARG (null) or EXT4PCF_E_CUDA; *centres is 0 before the first call. */
+EXT4PCF_API int ext4pcf_sector_centres(ext4pcf_ctx* ctx, int64_t* centres);
+
 /* Message of the last failure on this context ("" if none).  Valid until the next call. */
 EXT4PCF_API const char* ext4pcf_last_error(const ext4pcf_ctx* ctx);
 

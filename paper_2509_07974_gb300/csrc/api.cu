@@ -301,6 +301,19 @@ int ext4pcf_synchronize(ext4pcf_ctx* ctx) {
   return r != EXT4PCF_OK ? r : rc;
 }
 
+int ext4pcf_sector_centres(ext4pcf_ctx* ctx, int64_t* centres) {
+  if (!ctx || !centres) return EXT4PCF_E_INVALID_ARG;
+  ctx->err.clear();
+  CK(cudaSetDevice(ctx->cfg.device));
+  unsigned long long n = 0;
+  if (ctx->counter.p) {
+    CK(cudaMemcpyAsync(&n, (unsigned long long*)ctx->counter.p + 1, 8, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+  }
+  *centres = (int64_t)n;
+  return EXT4PCF_OK;
+}
+
 }  // extern "C"
 
 namespace {
@@ -433,7 +446,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   };
   int t_grid0 = -1;
   ENSURE(ctx->counter, 16);
-  CK(cudaMemsetAsync(ctx->counter.p, 0, 8, s));
+  CK(cudaMemsetAsync(ctx->counter.p, 0, 16, s));  // pairs, centres through angular sectors
   const bool tc = prec == EXT4PCF_TF32 || prec == EXT4PCF_SPLIT_BF16 || prec == EXT4PCF_3XTF32 ||
                   prec == EXT4PCF_SPLIT_F16;
   // waves that pack the centres of several catalogues: the split-FP16 contraction, the gather
@@ -1159,7 +1172,7 @@ int ext4pcf_measure3(ext4pcf_ctx* ctx, const double* positions, const double* sh
   bins.rmax = radial_bins[n_bins];
   // ---- grid (FP64 sorted catalogue)
   ENSURE(ctx->counter, 16);
-  CK(cudaMemsetAsync(ctx->counter.p, 0, 8, s));
+  CK(cudaMemsetAsync(ctx->counter.p, 0, 16, s));  // pairs, centres through angular sectors
   ENSURE(ctx->bbox, (4 + 4 * 512) * 8);
   ENSURE(ctx->geom, sizeof(GridGeom));
   CK(grid_bbox(positions, nk, (double*)ctx->bbox.p, s));

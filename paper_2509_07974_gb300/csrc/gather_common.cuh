@@ -127,7 +127,7 @@ struct GatherArgs {
   int cap;
   int mb;    // powers per warp block (<= MB)
   int nblk;  // power blocks
-  unsigned long long* pair_count;
+  unsigned long long* pair_count;  // [0]: pairs, [1]: centres that gather_sector took
   float dense_min;  // FP32: centres of catalogues at least this dense go to gather_sector (0: none)
 };
 

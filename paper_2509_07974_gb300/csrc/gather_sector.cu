@@ -832,7 +832,10 @@ gather_sector_kernel(const __grid_constant__ SectorArgs args, float2* __restrict
         xw[2 * (size_t)c + 1] = make_float2(ww, 0.f);
       }
     }
-    if (tid == 0) atomicAdd(ga.pair_count, pairs_here);
+    if (tid == 0) {
+      atomicAdd(ga.pair_count, pairs_here);
+      atomicAdd(ga.pair_count + 1, 1ull);  // centres of this kernel
+    }
   }
 }
 

@@ -3,7 +3,8 @@
 The functions ``ext4pcf_create``, ``ext4pcf_destroy``, ``ext4pcf_measure``,
 ``ext4pcf_to_real_space``, ``ext4pcf_to_map4``, ``ext4pcf_to_real_space_noalloc``,
 ``ext4pcf_map_direct``, ``ext4pcf_measure3``, ``ext4pcf_nth_order_components``, ``ext4pcf_nth_order_factors``,
-``ext4pcf_contraction_tables``, ``ext4pcf_synchronize`` and ``ext4pcf_last_error`` mirror the C ABI one to one; pointer arguments accept torch tensors (device or host), numpy arrays, raw
+``ext4pcf_contraction_tables``, ``ext4pcf_sector_centres``, ``ext4pcf_synchronize`` and
+``ext4pcf_last_error`` mirror the C ABI one to one; pointer arguments accept torch tensors (device or host), numpy arrays, raw
 integer addresses or None.  ``Estimator`` wraps them for torch users: it allocates outputs
 and passes the current CUDA stream.  Every computation happens in the CUDA library; there
 is no fallback, and loading fails loudly if the library has not been built.
@@ -83,7 +84,8 @@ def load(path: str = LIB_PATH):
     lib.ext4pcf_synchronize.restype = I
     lib.ext4pcf_last_error.argtypes = [P]
     lib.ext4pcf_last_error.restype = ctypes.c_char_p
-    for f in ("ext4pcf_create", "ext4pcf_destroy", "ext4pcf_measure", "ext4pcf_measure_batch", "ext4pcf_multipoles",
+    lib.ext4pcf_sector_centres.argtypes = [P, ctypes.POINTER(I64)]
+    for f in ("ext4pcf_create", "ext4pcf_destroy", "ext4pcf_sector_centres", "ext4pcf_measure", "ext4pcf_measure_batch", "ext4pcf_multipoles",
               "ext4pcf_to_real_space",
               "ext4pcf_to_map4", "ext4pcf_map_direct"):
         getattr(lib, f).restype = I
@@ -164,6 +166,13 @@ def ext4pcf_multipoles(ctx, positions, shears, weights, n_gal, radial_bins, n_bi
                                    _addr(radial_bins), int(n_bins), int(n_max), _addr(centres), int(n_centres),
                                    _addr(records))
     return _check(ctx, rc)
+
+
+def ext4pcf_sector_centres(ctx) -> int:
+    """Centres of the last call that the FP32 gather summed through angular sectors."""
+    n = ctypes.c_int64()
+    _check(ctx, load().ext4pcf_sector_centres(ctx, ctypes.byref(n)))
+    return n.value
 
 
 def record_layout(n_bins, n_max):
