@@ -886,18 +886,34 @@ cudaError_t gather_sector(const SortedCat& cat, const SortedCat& cen, const Bins
   if (fixed + 2 * slot > budget) return cudaSuccess;
   a.slots = (int)std::min<size_t>(kSlots, (budget - fixed) / slot);
   const double rm2 = g.bins.rmax * g.bins.rmax;
-  double rest = 0.0;  // part of the candidates in bins that get no sectors
-  for (int b = 31, n = 0; b >= 0; --b) {
-    a.share[b] = b < g.bins.nb ? (float)(0.9 * (g.bins.e2[b + 1] - g.bins.e2[b]) / rm2) : 0.f;
-    if (a.share[b] > 0.f && ++n > a.slots) rest += a.share[b];
+  double rest = 0.0, covered = 0.0;  // parts of the candidates in bins that get no sectors, in any bin
+  int sectored = 0;
+  for (int b = 31; b >= 0; --b) {
+    const double part = b < g.bins.nb ? (g.bins.e2[b + 1] - g.bins.e2[b]) / rm2 : 0.0;
+    a.share[b] = (float)(0.9 * part);
+    covered += part;
+    if (part > 0.0 && ++sectored > a.slots) rest += part;
   }
-  // Which catalogues.  Clocks per centre, measured: gather.cu 6.4 + 0.165 powers a candidate (11.8 at
-  // n_max = 13, 12.5 at 15, 14.1 at 20, about twice this kernel's at 30); here 9.6 and 30 for each in a bin without
-  // sectors, and 25000 a centre for the moments' transform and the like.  So at ten bins over two
-  // decades from 6600 candidates on at n_max = 20, 3200 at 30, and never below n_max = 9.
-  const double gain = 6.4 + 0.165 * (L.max_pow + 1) - (9.6 + 30.0 * rest);
+  sectored = std::min(sectored, a.slots);
+  // Which catalogues.  Clocks per centre, measured on few bins beside the sectored ones: gather.cu 6.4 +
+  // 0.165 powers a candidate; here 9.6 and 27 for each in a bin without sectors, and 25000 a centre for
+  // the moments' transform and the like.  At ten bins from 0.5 to 40 the line is 6670 candidates at
+  // n_max = 20 and 4230 at 30; at most four bins 27000 at n_max = 9, 42000 at 8, 94300 at 7, and no catalogue
+  // below.  Records of 1216 centres just past it, gather.cu and here: 0.541, 0.526 ms (n_max = 20, 4 bins),
+  // 1.98, 1.84 ms (8, 4), 4.23, 3.74 ms (7, 4).
+  const int npow = L.max_pow + 1;
+  const double gain = 6.4 + 0.165 * npow - (9.6 + 27.0 * rest);
   if (gain <= 0.0) return cudaSuccess;
-  const double least = 25000.0 / gain;
+  // Raised, or no catalogue, where by a second fit (916 cases: n_max 7 to 40, 1 to 16 bins, outer to inner radius 2
+  // to 80; rms 5%) gather.cu is the faster one at the line: narrow bins leave many pairs without sectors,
+  // whose sums cost by the power block (n_max = 40, ten bins to a twentieth of the radius, two of them sectored,
+  // 8450 candidates: 1.39 ms there, 1.64 ms here), and many powers or few pairs among the candidates move
+  // it up.
+  const double there = 0.98 * (4.3 + covered * nblk * (mb == kMB ? 1.5 : 2.1));
+  const double here = 5.0 + 0.2 * K * covered + 0.47 * sectored + rest * (25.0 + 4.3 * nblk);
+  if (here >= there) return cudaSuccess;
+  const double once = 29700.0 + 300.0 * L.nb * nblk + 6.8 * sectored * K * npow - 0.98 * (13800.0 + 420.0 * L.nb * nblk);
+  const double least = std::max(25000.0 / gain, once / (there - here));
   if (cat.n < least) return cudaSuccess;
   g.dense_min = *dense_min = (float)least;
   const size_t smem = fixed + a.slots * slot;

@@ -59,6 +59,24 @@ def test_dense_catalogues_go_through_sectors(torch_cuda, nmax, nb, n, side, dens
     assert taken == (len(centres) if dense else 0)
 
 
+@pytest.mark.parametrize("nmax,nb,n,inner", [(21, 10, 60000, 0.05), (24, 10, 20000, 0.05), (30, 10, 9000, 0.05),
+                                             (40, 10, 9000, 0.05), (18, 6, 29000, 0.3), (20, 12, 28000, 0.05)])
+def test_narrow_bins_stay_with_the_power_sums(torch_cuda, nmax, nb, n, inner):  # noqa: F811
+    """Many pairs in bins without sectors: the sector kernel was 3 to 18% slower there."""
+    cat, edges = _catalogue(n, 10.0, nmax + nb), np.geomspace(7.0 * inner, 7.0, nb + 1)
+    _, taken = _records(torch_cuda, "fp32", cat, edges, nmax, np.arange(7, dtype=np.int64))
+    assert taken == 0
+
+
+@pytest.mark.parametrize("nmax,n", [(7, 100000), (8, 45000), (9, 29000)])
+def test_lowest_orders_of_the_sectors(torch_cuda, nmax, n):  # noqa: F811
+    cat, edges = _catalogue(n, 10.0, nmax), np.geomspace(0.1, 7.0, 5)
+    centres = np.arange(12, dtype=np.int64) * (n // 12)
+    got, taken = _records(torch_cuda, "fp32", cat, edges, nmax, centres)
+    assert taken == 12
+    _within_rounding(torch_cuda, cat, edges, nmax, centres, got)
+
+
 @pytest.mark.parametrize("nmax,nb,n", [(20, 9, 11000), (30, 6, 9000)])
 def test_more_centres_than_blocks(torch_cuda, nmax, nb, n):  # noqa: F811
     cat, edges = _catalogue(n, 12.0, n), np.geomspace(0.1, 8.4, nb + 1)
