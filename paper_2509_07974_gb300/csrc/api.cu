@@ -18,13 +18,13 @@ cudaError_t scan_exclusive(unsigned* data, size_t n, unsigned* tmp, cudaStream_t
 cudaError_t real_space(const double* ups, int nb, int N, int nphi, double* gamma, double* norm,
                        double* scratch_norm, double* E_scratch, cudaStream_t s);
 size_t real_space_smem(int N, int nphi);
-int map4_nsplit(int chunk_tri, int ntri, int n_ap);
+int map4_nsplit(int chunk_tri, int ntri, int n_ap, int sms);
 cudaError_t map4_partials(const double* ups, const double* edges_host, int nb, int N, int nphi,
                           const double* ap_host, int n_ap, double* E_scratch, double* norm_chunk,
                           double* gam_chunk, double* tables, int chunk_tri, int nsplit, double* partial,
                           cudaStream_t s);
 size_t map4_table_bytes(int chunk_tri, int nphi, int n_ap);
-int map4_chunk(int ntri, int nphi, int n_ap);
+int map4_chunk(int ntri, int nphi, int n_ap, int sms);
 cudaError_t map4_finish_launch(const double* partial, int ntri, int n_ap, const double* d_xipm,
                                const double* d_tb, const double* d_area, int nb, const double* d_ap,
                                double* d_m4, double* d_eb, double* d_disc, cudaStream_t s);
@@ -1097,12 +1097,12 @@ int ext4pcf_to_map4(ext4pcf_ctx* ctx, const double* upsilon, const double* radia
   cudaStream_t s = ctx->stream;
   const int ntri = n_bins * n_bins * n_bins;
   const size_t nph2 = (size_t)n_phi * n_phi;
-  const int chunk = map4_chunk(ntri, n_phi, n_ap);
+  const int chunk = map4_chunk(ntri, n_phi, n_ap, ctx->sm_count);
   ENSURE(ctx->t_norm, (size_t)chunk * nph2 * 8);
   ENSURE(ctx->t_gam, (size_t)chunk * nph2 * 8 * 16);
   ENSURE(ctx->t_E, (size_t)(2 * n_max + 1) * n_phi * 16);
   ENSURE(ctx->t_tab, map4_table_bytes(chunk, n_phi, n_ap));
-  const int nsplit = map4_nsplit(chunk, ntri, n_ap);
+  const int nsplit = map4_nsplit(chunk, ntri, n_ap, ctx->sm_count);
   ENSURE(ctx->t_part, (size_t)ntri * nsplit * n_ap * 8 * 16);
   // small buffer: xi_acc [nb*6], tb [nb], area [nb], ap [n_ap], m4 [n_ap*16], eb [n_ap*16], disc [n_ap*16]
   const size_t small = (size_t)n_bins * 8 + n_ap * 49;

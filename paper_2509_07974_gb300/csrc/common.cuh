@@ -103,6 +103,14 @@ struct SortedCat {
   const float4* s4;       // (x_re, x_im, w, 0) as float
 };
 
+// SMs of the current device: the grids of persistent kernels and the rounds of blocks follow it
+inline int device_sms() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 1;
+}
+
 // kernels launched by this host thread (each launcher adds what it enqueues)
 extern thread_local long long g_launches;
 

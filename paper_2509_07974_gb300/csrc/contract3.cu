@@ -251,7 +251,7 @@ cudaError_t contract3_wave(const Layout& L, const Cx* rec, const Cx* xw, int T, 
   if (e != cudaSuccess) return e;
   contract3_kernel<Cx><<<(L.N + 1) * S * chunks, kC3Threads, smem, s>>>(L, t, rec, xw, T, S, chunks, scratch);
   const int total = 5 * (2 * L.N + 1) * nb2;
-  contract3_sum<<<std::min(4 * 152, (total + 127) / 128), 128, 0, s>>>(L, t, S, scratch, ups3);
+  contract3_sum<<<std::min(4 * device_sms(), (total + 127) / 128), 128, 0, s>>>(L, t, S, scratch, ups3);
   g_launches += 2;
   return cudaGetLastError();
 }

@@ -859,7 +859,7 @@ cudaError_t launch(SectorArgs& a, size_t smem, float2* rec, float2* xw, cudaStre
   for (int n = 0; n <= a.g.L.max_pow; ++n) jacobi_anger(n * kDeltaMax, K, a.coef + n * K);
   cudaError_t e = cudaFuncSetAttribute(gather_sector_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  gather_sector_kernel<K><<<std::min(a.g.plan.total, 152), kThreads, smem, s>>>(a, rec, xw);
+  gather_sector_kernel<K><<<std::min(a.g.plan.total, device_sms()), kThreads, smem, s>>>(a, rec, xw);
   ++g_launches;
   return cudaGetLastError();
 }

@@ -407,19 +407,19 @@ size_t map4_table_bytes(int chunk_tri, int nphi, int n_ap) {
 
 // Radial triples of one chunk: 256 MB of Gamma and tables, and whole rounds of two blocks per SM of
 // real_space_kernel (8 blocks a triple) where that leaves at least one.
-int map4_chunk(int ntri, int nphi, int n_ap) {
+int map4_chunk(int ntri, int nphi, int n_ap, int sms) {
   const size_t per = (size_t)nphi * nphi * 8 * sizeof(double2) + (size_t)3 * nphi * n_ap * sizeof(double);
   const size_t fit = std::max<size_t>(1, (size_t)(256u << 20) / per);
   if (fit >= (size_t)ntri) return ntri;
-  constexpr int kRound = 2 * 152 / 8;
-  return fit < kRound ? (int)fit : (int)(fit / kRound * kRound);
+  const size_t round = std::max(1, 2 * sms / 8);
+  return fit < round ? (int)fit : (int)(fit / round * round);
 }
 
 // Aperture measures: triples processed in chunks; returns per-(triple, slice, aperture)
 // partial sums in `partial` [ntri][nsplit][n_ap][8] complex, the angular bins of each
 // triple split into nsplit slices: 8 as the real-space blocks of the triple, more for a small chunk.
-int map4_nsplit(int chunk_tri, int ntri, int n_ap) {
-  int ns = std::max(8, (4 * 152 + chunk_tri - 1) / chunk_tri);
+int map4_nsplit(int chunk_tri, int ntri, int n_ap, int sms) {
+  int ns = std::max(8, (4 * sms + chunk_tri - 1) / chunk_tri);
   const size_t cap = (size_t)(256u << 20) / ((size_t)ntri * n_ap * 8 * 16);
   if ((size_t)ns > cap) ns = (int)cap;
   return ns < 1 ? 1 : (ns > 16 ? 16 : ns);
