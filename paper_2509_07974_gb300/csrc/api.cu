@@ -821,11 +821,15 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   }
   ENSURE(ctx->xw, (size_t)Tmax * 2 * cbytes);
   std::vector<float> trial_ms;
-  const size_t corr_doubles = corrections_slot_doubles(L, n_out);
-  ENSURE(ctx->corr, corr_doubles * 8 * n_out);
-  CK(cudaMemsetAsync(ctx->corr.p, 0, corr_doubles * 8 * n_out, s));
+  // correction sums of the slots that are live at once: all of them, or the CUDA-core forms' one
+  const int corr_slots = records ? 0 : cc ? 1 : n_out;
+  const size_t corr_doubles = records ? 0 : corrections_slot_doubles(L, corr_slots);
+  if (!records) {
+    ENSURE(ctx->corr, corr_doubles * 8 * corr_slots);
+    CK(cudaMemsetAsync(ctx->corr.p, 0, corr_doubles * 8 * corr_slots, s));
+  }
   const size_t red_doubles = h16 ? 2 * ctx->basis.elems() : tc ? tc_reduced_doubles(L) : 0;
-  if (tc) {
+  if (tc && !records) {
     ENSURE(ctx->tc_red, red_doubles * 8 * n_out);
     CK(cudaMemsetAsync(ctx->tc_red.p, 0, red_doubles * 8 * n_out, s));
   }
@@ -884,12 +888,11 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
   int red_slot = -1;  // output slot of the CUDA-core forms' reduced array
   // its sums and their multiple-counting terms to its output, and the arrays cleared for the next
   auto flush_slot = [&]() -> cudaError_t {
-    double* corr = corr_base + corr_doubles * (size_t)red_slot;
-    cudaError_t e = corrections_finish(L, n_out, red_slot, 1, corr_base, d_xi, s);
+    cudaError_t e = corrections_finish(L, 1, corr_base, d_xi ? d_xi + (size_t)red_slot * 6 * n_bins : nullptr, s);
     if (e == cudaSuccess)
-      e = basis_expand(ctx->basis, red_base, cc_slices, corr, d_ups + 2 * ups_elems * (size_t)red_slot, s);
+      e = basis_expand(ctx->basis, red_base, cc_slices, corr_base, d_ups + 2 * ups_elems * (size_t)red_slot, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(red_base, 0, cc_bytes, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(corr, 0, corr_doubles * 8, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(corr_base, 0, corr_doubles * 8, s);
     return e;
   };
   for (;;) {
@@ -926,9 +929,12 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
       continue;
     }
     if (timing) t_w1 = tmark();
-    if (cc && g0.slot != red_slot) {  // the next slot: the last one's sums go to its output
-      if (red_slot >= 0) CK(flush_slot());
-      red_slot = g0.slot;
+    if (cc) {
+      if (g0.slot != red_slot) {  // the next slot: the last one's sums go to its output
+        if (red_slot >= 0) CK(flush_slot());
+        red_slot = g0.slot;
+      }
+      P.seg[0].slot = 0;  // (the wave's one segment: of the correction sums)
     }
     if (f64) {
       CK(contract_wave<double>(L, ctx->basis, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, g0.t, g0.n_live,
@@ -948,9 +954,9 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
     }
     if (timing) t_w2 = tmark();
     if (f64) {
-      CK(corrections_wave<double>(L, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, P, n_out, corr_base, d_xi != nullptr, s));
+      CK(corrections_wave<double>(L, (const double2*)ctx->rec.p, (const double2*)ctx->xw.p, P, corr_slots, corr_base, d_xi != nullptr, s));
     } else {
-      CK(corrections_wave<float>(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, n_out, corr_base, d_xi != nullptr, s));
+      CK(corrections_wave<float>(L, (const float2*)ctx->rec.p, (const float2*)ctx->xw.p, P, corr_slots, corr_base, d_xi != nullptr, s));
     }
     if (timing) {
       const int t_w3 = tmark();
@@ -980,7 +986,7 @@ int measure_impl(ext4pcf_ctx* ctx, const double* positions, const double* shears
     CK(cudaMemcpyAsync(rec_out, ctx->rec_out.p, (size_t)n_rec * L.rec * 16, cudaMemcpyDeviceToHost, s));
   if (red_slot >= 0) CK(flush_slot());
   // ---- per output slot: every ordered triple from the reduced array, less the corrections
-  if (tc && !records) CK(corrections_finish(L, n_out, 0, n_out, corr_base, d_xi, s));
+  if (tc && !records) CK(corrections_finish(L, n_out, corr_base, d_xi, s));
   for (int o = 0; o < n_out && tc && !records; ++o) {
     double* ups_o = d_ups + 2 * ups_elems * (size_t)o;
     const double* corr_o = corr_base + corr_doubles * (size_t)o;

@@ -258,13 +258,12 @@ cudaError_t contract_wave(const Layout& L, const Basis& B, const cplx_t<R>* rec,
                           const int* n_live, int w0, double* red, cudaStream_t s);
 
 // corrections.cu: the multiple-counting sums (and xi accumulators) of every segment into its slot's
-// copies, corr + slot * corrections_slot_doubles; finish adds the copies of `count` slots into the
-// first one each and their xi sums into xi [n_out][nb][3][2] (if non-null)
+// copies, corr + slot * corrections_slot_doubles; finish adds the copies of every slot into the
+// first one and their xi sums into xi [n_out][nb][3][2] (if non-null)
 template <typename R>
 cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t<R>* xw, const WavePlan& plan, int n_out,
                              double* corr, bool xi, cudaStream_t s);
-cudaError_t corrections_finish(const Layout& L, int n_out, int first, int count, double* corr, double* xi,
-                               cudaStream_t s);
+cudaError_t corrections_finish(const Layout& L, int n_out, double* corr, double* xi, cudaStream_t s);
 size_t corrections_slot_doubles(const Layout& L, int n_out);
 
 // contract_tc.cu (tensor cores).  The wave is contracted into the reduced array of the

@@ -248,12 +248,16 @@ __global__ void corrections_sum(const CorrLayout C, int copies, size_t slot_stri
 
 }  // namespace
 
-// copies per slot: slices enough to fill the SMs from one sg each while the slots are few; with
-// many slots a wave's segments are short, and the copies would take more memory than the outputs'
-// former sums
-int corrections_copies(int n_out) { return n_out <= 8 ? 16 : n_out < 32 ? 4 : 2; }
+// Copies per slot, of n_out slots that are summed at once: slices enough to fill the SMs from one sg each while the
+// slots are few (with many a wave's segments are short), and no more than two where all of them would
+// take over 128 MB (16 copies of 8 slots are 56 MB at n_max = 20, 10 bins, 2.25 GB at 40, 32).
+static int corrections_copies(const CorrLayout& C, int n_out) {
+  const size_t fit = ((size_t)128 << 20) / (C.elems * sizeof(double2) * (size_t)n_out);
+  return (int)std::min<size_t>(n_out <= 8 ? 16 : n_out < 32 ? 4 : 2, std::max<size_t>(fit, 2));
+}
 size_t corrections_slot_doubles(const Layout& L, int n_out) {
-  return 2 * CorrLayout::make(L.N, L.nb).elems * corrections_copies(n_out);
+  const CorrLayout C = CorrLayout::make(L.N, L.nb);
+  return 2 * C.elems * corrections_copies(C, n_out);
 }
 
 template <typename R>
@@ -267,18 +271,18 @@ cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t
   const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>), (size_t)threads * 4 * sizeof(double2));
   cudaError_t e = cudaFuncSetAttribute(corrections_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  corrections_kernel<R><<<dim3(C.nsig + 2 * L.N + 2, corrections_copies(n_out)), threads, smem, s>>>(
-      L, C, rec, xw, plan, reinterpret_cast<double2*>(corr), C.elems * corrections_copies(n_out), xi);
+  const int copies = corrections_copies(C, n_out);
+  corrections_kernel<R><<<dim3(C.nsig + 2 * L.N + 2, copies), threads, smem, s>>>(
+      L, C, rec, xw, plan, reinterpret_cast<double2*>(corr), C.elems * copies, xi);
   ++g_launches;
   return cudaGetLastError();
 }
 
-cudaError_t corrections_finish(const Layout& L, int n_out, int first, int count, double* corr, double* xi,
-                               cudaStream_t s) {
+cudaError_t corrections_finish(const Layout& L, int n_out, double* corr, double* xi, cudaStream_t s) {
   const CorrLayout C = CorrLayout::make(L.N, L.nb);
-  const int copies = corrections_copies(n_out);
-  for (int o = first; o < first + count; o += 32768) {
-    const int n = std::min(32768, first + count - o);
+  const int copies = corrections_copies(C, n_out);
+  for (int o = 0; o < n_out; o += 32768) {
+    const int n = std::min(32768, n_out - o);
     corrections_sum<<<dim3((unsigned)((C.elems + 255) / 256), n), 256, 0, s>>>(
         C, copies, C.elems * copies, reinterpret_cast<double2*>(corr) + (size_t)o * C.elems * copies,
         xi ? xi + (size_t)o * 6 * L.nb : nullptr);
