@@ -43,7 +43,8 @@ __device__ __forceinline__ bool corr_valid(const Layout& L, int k, int sg) {
   return p && basis_in_g(N, basis_col_index(q, sg));
 }
 
-template <typename R>
+// SHARED: tiles that several threads share (up to eight bins)
+template <typename R, bool SHARED>
 __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const CorrLayout C,
                                                           const cplx_t<R>* __restrict__ rec,
                                                           const cplx_t<R>* __restrict__ xw,
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
   const int sg = wk ? job - C.nsig : -2 * N - 6 + job;  // (W blocks: the index c)
   const int width = (wk ? 2 : 6) * nbp;                 // staged values per centre
   const int tiles = (wk ? 1 : 6) * nt * nt;
-  const int run = sizeof(R) == 4 ? corr_run(nb) : 16;
+  const int run = SHARED && sizeof(R) == 4 ? corr_run(nb) : 16;
   Cx* st = reinterpret_cast<Cx*>(smem_raw);  // [kCorrChunk][width]
   // the value this thread stages of every (blockDim / width)-th centre: its place in a record (-1: a
   // zero), its conjugation and its centre factor (0: none, 1: x, 2: x^*, 3: w)
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
       }
     }
   }
-  const int parts = max(1, min(kCorrParts, (int)blockDim.x / tiles));
+  const int parts = SHARED ? max(1, min(kCorrParts, (int)blockDim.x / tiles)) : 1;
   for (int i0 = 0; i0 < tiles; i0 += blockDim.x) {
     const int tile = parts > 1 ? tid % tiles : i0 + tid, part = parts > 1 ? tid / tiles : 0;
     const int k = tile / (nt * nt), ta = 2 * ((tile / nt) % nt), tb = 2 * (tile % nt);
@@ -267,12 +268,15 @@ cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t
   const CorrLayout C = CorrLayout::make(L.N, L.nb);
   const int nt = (L.nb + 1) / 2;
   // up to eight bins 192 threads: 8, 8, 3 and 2 to a tile of the six X arrays
-  const int threads = std::min(384, std::max(nt <= 4 ? 192 : 160, (6 * nt * nt + 31) / 32 * 32));
-  const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>), (size_t)threads * 4 * sizeof(double2));
-  cudaError_t e = cudaFuncSetAttribute(corrections_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const bool shared = nt <= 4;
+  const int threads = std::min(384, std::max(shared ? 192 : 160, (6 * nt * nt + 31) / 32 * 32));
+  const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>),
+                               (size_t)threads * (shared ? 4 : 1) * sizeof(double2));
+  auto kernel = shared ? corrections_kernel<R, true> : corrections_kernel<R, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int copies = corrections_copies(C, n_out);
-  corrections_kernel<R><<<dim3(C.nsig + 2 * L.N + 2, copies), threads, smem, s>>>(
+  kernel<<<dim3(C.nsig + 2 * L.N + 2, copies), threads, smem, s>>>(
       L, C, rec, xw, plan, reinterpret_cast<double2*>(corr), C.elems * copies, xi);
   ++g_launches;
   return cudaGetLastError();
