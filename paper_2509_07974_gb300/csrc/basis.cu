@@ -213,7 +213,7 @@ cudaError_t basis_expand(const Basis& B, const double* red, int slices, const do
   double2* u = reinterpret_cast<double2*>(ups);
   const size_t smem = (size_t)(3 * B.nb * B.nb + B.nb) * sizeof(double2);
   auto kernel = slices > 1 ? expand_kernel<true> : expand_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kernel);
   if (e != cudaSuccess) return e;
   kernel<<<blocks, kExpandThreads, smem, s>>>(B, r, slices, c, inv, u);
   ++g_launches;

@@ -111,6 +111,14 @@ inline int device_sms() {
   return n > 0 ? n : 1;
 }
 
+// Dynamic shared memory for a kernel, always up to the device's limit (none of the kernels that take
+// it has static shared memory): the attribute belongs to the kernel, so a launcher that set what its own
+// sizes need could lower it between another host thread's setting and launch, which then failed.
+template <typename K>
+inline cudaError_t allow_smem(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+
 // kernels launched by this host thread (each launcher adds what it enqueues)
 extern thread_local long long g_launches;
 

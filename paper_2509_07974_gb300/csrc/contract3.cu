@@ -247,7 +247,7 @@ cudaError_t contract3_wave(const Layout& L, const Cx* rec, const Cx* xw, int T, 
   // components that 512 consecutive sums touch, at most
   const int items = std::min(t.nitem, (outs + nb2 - 2) / nb2 + 1);
   const size_t smem = (size_t)kC3Centres * items * 2 * L.nb * sizeof(double2);
-  cudaError_t e = cudaFuncSetAttribute(contract3_kernel<Cx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(contract3_kernel<Cx>);
   if (e != cudaSuccess) return e;
   contract3_kernel<Cx><<<(L.N + 1) * S * chunks, kC3Threads, smem, s>>>(L, t, rec, xw, T, S, chunks, scratch);
   const int total = 5 * (2 * L.N + 1) * nb2;

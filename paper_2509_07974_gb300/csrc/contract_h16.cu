@@ -6,9 +6,9 @@
 // over the centres.  Every row product serves four families, so 1643 tiles of 128 rows (n_max = 20,
 // 10 bins) hold what took 5572 tiles with a row type per component.  Forming the rows on the CUDA
 // cores is the larger part of the work.  One wave of 8192 centres at these sizes: 6.5 -> 2.24 ms
-// (3300 clocks per 64-centre stage of a tile, of which shared memory is busy for about 2750: row
-// products read 1024 wavefronts, the columns' embedding moves 480, the MMAs read 480 and the bulk
-// copies write 480).  The data are arranged for the producers:
+// (3300 clocks per 64-centre stage of a tile; by count of its accesses shared memory is busy for about 2750
+// of them: row products read 1024 wavefronts, the columns' embedding moves 480, the MMAs read 480
+// and the bulk copies write 480).  The data are arranged for the producers:
 //  * Power-of-two row scales.  A pre-pass finds the largest |component| of every row of the
 //    wave array and the transpose writes each row times 2^k, its largest component in
 //    [2^6, 2^7).  A product of two rows is then below 2^15, inside the fp16 range, with no
@@ -736,8 +736,7 @@ size_t h_smem_bytes(int nb) { return h_fixed_smem(nb) + (size_t)h_in_stages(nb) 
 
 template <int CW, int SLOTS>
 cudaError_t launch_h16(const HArgs& a, int sms, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(contract_h16_kernel<CW, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(contract_h16_kernel<CW, SLOTS>);
   if (e != cudaSuccess) return e;
   contract_h16_kernel<CW, SLOTS><<<sms, kHThreads, smem, s>>>(a);
   ++g_launches;

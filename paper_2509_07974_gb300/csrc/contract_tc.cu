@@ -654,7 +654,7 @@ size_t tc_smem_bytes(int nb, int N, int prec) {
 
 template <int PREC>
 cudaError_t launch_tc(const TcArgs& a, const CUtensorMap& tm, size_t smem, int sms, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(contract_tc_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(contract_tc_kernel<PREC>);
   if (e != cudaSuccess) return e;
   contract_tc_kernel<PREC><<<sms, kThreads, smem, s>>>(a, tm);
   return cudaGetLastError();

@@ -273,7 +273,7 @@ cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t
   const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>),
                                (size_t)threads * (shared ? 4 : 1) * sizeof(double2));
   auto kernel = shared ? corrections_kernel<R, true> : corrections_kernel<R, false>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kernel);
   if (e != cudaSuccess) return e;
   const int copies = corrections_copies(C, n_out);
   kernel<<<dim3(C.nsig + 2 * L.N + 2, copies), threads, smem, s>>>(

@@ -445,7 +445,7 @@ cudaError_t gather_wave32(const SortedCat& cat, const SortedCat& cen, const Bins
   if (cap > 8192) cap = 8192;
   a.cap = cap;
   const size_t smem = fixed + (size_t)cap * per_pair;
-  cudaError_t e = cudaFuncSetAttribute(gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(gather_kernel);
   if (e != cudaSuccess) return e;
   a.dense_min = 0.f;
   e = gather_sector(cat, cen, bins, L, plan, accumulate, a.mb, a.nblk, rec, xw, pair_count, s, &a.dense_min);

@@ -369,7 +369,7 @@ cudaError_t gather_wave64(const SortedCat& cat, const SortedCat& cen, const Bins
   if (cap > 8192) cap = 8192;
   a.cap = cap;
   const size_t smem = fixed + (size_t)cap * per_pair;
-  cudaError_t e = cudaFuncSetAttribute(gather64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(gather64_kernel);
   if (e != cudaSuccess) return e;
   gather64_kernel<<<plan.total, kThreads, smem, s>>>(a, rec, xw);
   ++g_launches;

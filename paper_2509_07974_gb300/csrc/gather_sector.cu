@@ -20,8 +20,8 @@
 // Measured: 8192 centres with 28000 candidates each, n_max = 20, 11.1 -> 8.0 ms; 256 centres of four
 // patches, n_max = 30, three passes of the tree approximation, 7.6 -> 3.6 ms.  The records' error
 // against 64 bits stays (7.1e-8 -> 6.9e-8 of the largest; 100000 galaxies, 7 bins, n_max = 15).  No
-// unit is saturated: with three warps to a scheduler the latencies of (a) and the unequal sectors of
-// (b) are what is left, issue slots half used.
+// unit is saturated: with three warps to a scheduler the latencies of (a), the unequal sectors
+// of (b) and the barriers between them are what is left.
 #include <algorithm>
 #include <cmath>
 
@@ -857,7 +857,7 @@ void jacobi_anger(double z, int K, float* out) {
 template <int K>
 cudaError_t launch(SectorArgs& a, size_t smem, float2* rec, float2* xw, cudaStream_t s) {
   for (int n = 0; n <= a.g.L.max_pow; ++n) jacobi_anger(n * kDeltaMax, K, a.coef + n * K);
-  cudaError_t e = cudaFuncSetAttribute(gather_sector_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(gather_sector_kernel<K>);
   if (e != cudaSuccess) return e;
   gather_sector_kernel<K><<<std::min(a.g.plan.total, device_sms()), kThreads, smem, s>>>(a, rec, xw);
   ++g_launches;

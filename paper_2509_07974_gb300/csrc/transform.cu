@@ -368,7 +368,7 @@ template <RealOut OUT>
 cudaError_t launch_real(int blocks, size_t smem, cudaStream_t s, const double2* U, int nb, int N, int nphi,
                         const double2* E, int tri0, int ntri, const double* norm_in, double* norm_out, double2* gam,
                         size_t stride) {
-  cudaError_t e = cudaFuncSetAttribute(real_space_kernel<OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(real_space_kernel<OUT>);
   if (e != cudaSuccess) return e;
   real_space_kernel<OUT><<<blocks, kRealThreads, smem, s>>>(U, nb, N, nphi, E, tri0, ntri, norm_in, norm_out, gam,
                                                             stride);
@@ -437,7 +437,7 @@ cudaError_t map4_partials(const double* ups, const double* edges_host, int nb, i
   const size_t smem4 = kM4Coef * kM4Row * sizeof(double2) + kM4Bins * (size_t)n_ap * sizeof(double);
   // (the sums at the end, [parts][n_ap][kM4Coef] with parts n_ap <= 8 or parts = 1, fit in it)
   static_assert(kM4Groups <= kM4Bins && 64 <= kM4Bins, "sums");
-  cudaError_t e = cudaFuncSetAttribute(map4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem4);
+  cudaError_t e = allow_smem(map4_kernel);
   if (e != cudaSuccess) return e;
   Map4Args a;
   a.nb = nb; a.nphi = nphi; a.n_ap = n_ap;
