@@ -99,6 +99,16 @@ def reduced_contraction_flop(n_centres, nmax, nb):
     return 8.0 * n_centres * per_centre
 
 
+def map4_launches(nb, n_phi, n_ap):
+    """Kernels of one ext4pcf_to_map4 call: the angle table, the angles' turns and the finish, and per chunk of
+    radial triples the reciprocal counts, Gamma, the exponential tables and the integrals.  A chunk (csrc/transform.cu)
+    is what 256 MB of Gamma and tables hold, in whole rounds of two real-space blocks per SM."""
+    per = n_phi * n_phi * 8 * 16 + 3 * n_phi * n_ap * 8
+    chunk, rnd = max(1, (256 << 20) // per), 2 * N_SM // 8
+    chunk = nb ** 3 if chunk >= nb ** 3 else chunk if chunk < rnd else chunk // rnd * rnd
+    return 3 + 4 * -(-nb ** 3 // chunk)
+
+
 class ClockSampler:
     """nvidia-smi clocks and throttle reasons sampled every 200 ms while running."""
 
@@ -608,11 +618,6 @@ def run_ours(args):
                "sample": "%d random centres of the %d-galaxy catalogue (all galaxies as neighbours), %d pairs, %.1f s"
                          % (args.oracle_centres, len(w), opairs, odt)}
 
-    # kernels per step: those of ext4pcf_measure (counted by the library) plus those of
-    # ext4pcf_to_map4: angle table + (norm, gamma, integrate) per chunk of radial triples + finish
-    nph2 = N_PHI * N_PHI
-    chunk = min(nb ** 3, max(1, (256 << 20) // (nph2 * 8 * 16)))
-    map4_launches = 2 + 3 * ((nb ** 3 + chunk - 1) // chunk)
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": "pairs/s", "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": dev_ms_max / args.steps, "higher_is_better": True,
@@ -635,7 +640,8 @@ def run_ours(args):
                 "cpu_baseline": cpu,
                 "next_rows": {"map_direct": direct, "third_order": third},
                 "clocks": clocks,
-                "gpu_launches": int((bd["launches"] + map4_launches) * args.steps)}
+                # kernels per step: those of ext4pcf_measure (counted by the library) and of ext4pcf_to_map4
+                "gpu_launches": int((bd["launches"] + map4_launches(nb, N_PHI, len(ap))) * args.steps)}
         print(json.dumps(line), flush=True)
     est.close()
 
@@ -886,7 +892,7 @@ def run_batched(args, kind):
                         "d2h_bytes_per_step": int(d2h)},
                 "roofline": roof_main, "roofline_secondary": roof_other, "cpu_baseline": cpu,
                 "clocks": clocks,
-                "gpu_launches": int(bd["launches"] * args.steps)}
+                "gpu_launches": int((bd["launches"] + (map4_launches(nb, N_PHI, len(ap)) if want_map4 else 0)) * args.steps)}
         if want_map4:
             line["map4_by_radius"] = {"%.2f" % ap[i]: float(m4[i, 0, 0]) for i in (0, len(ap) // 2, len(ap) - 1)}
         if tree_info is not None:
