@@ -79,8 +79,52 @@ def gather_flop_per_pair(nmax):
     return 8 * (4 * N + 3) + 8 * (4 * N + 5) + 4 * ((2 * N + 1) + (2 * N + 3) + (2 * N + 1)) + 6 * (2 * N + 6) + 40
 
 
-GATHER_NOTE = ("the sums taken power by power; dense catalogues are summed through angular sectors (csrc/gather_sector.cu), "
-               "which executes about a fifth of these operations, so frac is not the FMA pipe's use")
+def sector_flop_per_pair(nmax):
+    """FP32 work of one pair in the sums of the sector gather (csrc/gather_sector.cu): seven weights times K
+    Chebyshev polynomials (the first is 1: additions), the recurrence, both halves of a packed instruction, and
+    ~50 for the weights and the triple terms.  The pairs of bins without sectors cost more and
+    finding the pairs is not in it, so a rate from this is a lower bound."""
+    K = 12 if 2 * nmax + 6 <= 46 else 16
+    return 7 + 18 * (K - 1) + 50
+
+
+def gather_roofline(pairs, nmax, sector_share, waves, ms, peak):
+    """Executed FP32 operations of the gather's sums against the FMA pipe; sector_share: part of the centres
+    that went through sectors.  (algorithmic_*: the same sums taken power by power.)"""
+    per_pair = gather_flop_per_pair(nmax)
+    executed = sector_share * sector_flop_per_pair(nmax) + (1.0 - sector_share) * per_pair
+    rate = lambda f: f * pairs / (ms / 1e3) / 1e12 if ms > 0 else None  # noqa: E731
+    return {"bound": "alu", "kernel": "gather_sector" if sector_share > 0.5 else "gather", "achieved": rate(executed),
+            "peak": peak, "unit": "TFLOP/s", "frac": (rate(executed) or 0.0) / peak, "traffic": None,
+            "ms_per_launch": ms / waves, "executed_flop_per_pair": executed, "sector_share": sector_share,
+            "algorithmic_flop_per_pair": per_pair, "algorithmic_tflops": rate(per_pair)}
+
+
+def basis_rows(nmax):
+    """Rows (sg, a) of the independent sums per sg (csrc/basis.cuh): those of F0..F3, which some component at
+    |n2|, |n3| <= nmax reads, then those of FW."""
+    lo, hi = {}, {}
+    for n2 in range(-nmax, nmax + 1):
+        for n3 in range(-nmax, nmax + 1):
+            for k in ((n2 + n3 - 3, -n2 - 2, -n3 - 3), (n2 + n3 - 1, -n2 - 2, -n3 - 1)):
+                for i in range(3):
+                    sg = sum(k) - k[i]
+                    rest = [k[j] for j in range(3) if j != i]
+                    lo[sg] = min([lo.get(sg, rest[0])] + rest)
+                    hi[sg] = max([hi.get(sg, rest[0])] + rest)
+    return [hi[s] - lo[s] + 1 for s in sorted(lo)], [2 * nmax + 1 - s for s in range(2 * nmax + 1)]
+
+
+def h16_mma_flop(n_centres, nmax, nb):
+    """MMA operations that the split-FP16 contraction issues: per 64 centres and tile of 128 rows 24 MMAs (three
+    products of the hi and lo halves) of K = 16 over the tile's columns, its padding included."""
+    pairs, groups = nb * (nb + 1) // 2, 1 if nb <= 12 else 2
+    rows = 64 if nb == 1 else 128
+    x, w = basis_rows(nmax)
+    tiles = lambda lens: sum(-(-n * pairs // rows) for n in lens)  # noqa: E731
+    pad = lambda families: (2 * families * nb + 15) // 16 * 16  # noqa: E731
+    columns = groups * tiles(x) * pad(4 // groups) + tiles(w) * pad(1)
+    return 24 * 2 * 128 * 16 * columns * n_centres / 64.0
 
 
 def contraction_flop(n_centres, nmax, nb):
@@ -97,6 +141,15 @@ def reduced_contraction_flop(n_centres, nmax, nb):
     n_sq = (2 * nmax + 1) ** 2
     per_centre = 8 * (n_sq + 4 * nmax + 1) * pairs * nb + n_sq * pairs * nb
     return 8.0 * n_centres * per_centre
+
+
+def issued_flop(precision, n_centres, nmax, nb):
+    """Operations that a form's contraction issues: all passes of the tensor-core forms."""
+    if precision == "f16x3":
+        return h16_mma_flop(n_centres, nmax, nb)
+    if precision in ("tf32", "3xtf32", "bf16x3"):
+        return (1 if precision == "tf32" else 3) * reduced_contraction_flop(n_centres, nmax, nb)
+    return contraction_flop(n_centres, nmax, nb)
 
 
 def map4_launches(nb, n_phi, n_ap):
@@ -525,21 +578,20 @@ def run_ours(args):
     h2d = hp.numel() * 8 + hs.numel() * 8 + hw.numel() * 8 + (hmask.numel() if hmask is not None else 0)
     d2h = m4.nbytes + eb.nbytes + disc.nbytes
 
+    sector_share = ext4pcf.ext4pcf_sector_centres(est.ctx) / max(1.0, bd["centres"])
+
     direct = third = None
     if rank == 0:
         direct = direct_estimator(est, tp, ts, tw, pos, sh, w, c["side"], dev, stream, flush, args,
                                   world == 1 and not args.no_baselines)
         third = third_order(dev, stream, flush, args)
 
-    # rooflines of the two dominant kernels, algorithmic FLOP per launch over the average
-    # launch duration in the timed steps.  Gather: FP32 work on the CUDA cores against the
-    # FP32 FMA pipe.  Contraction: complex multiply-adds of the outputs on the tensor cores
-    # against the TF32 rate (measured sustained bf16 x the nominal tf32/bf16 ratio 1.1/2.25;
-    # the 3xTF32 form issues three MMAs per algorithmic product).
+    # rooflines of the two dominant kernels: the operations they execute over their time in the timed
+    # steps (algorithmic_*: the operations of the plain sums, more than are executed).  Gather: FP32 work on
+    # the CUDA cores against the FP32 FMA pipe.  Contraction: the MMAs issued, against the rate
+    # of their operand type.
     waves = max(1, bd["waves"])
-    flop_pair = gather_flop_per_pair(nmax)
     g_ms = bd["ms_gather"] / waves
-    g_ach = flop_pair * pairs / waves / (g_ms / 1e3) / 1e12
     fp32_peak = N_SM * FP32_LANES_PER_SM * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
     tc_form = args.precision in ("tf32", "3xtf32", "bf16x3", "f16x3")
     c_flop_full = contraction_flop(bd["centres"], nmax, nb)
@@ -551,15 +603,16 @@ def run_ours(args):
     # the measured bf16 rate, kind::tf32 at that rate times the nominal ratio 1.1/2.25
     f16_kind = args.precision in ("f16x3", "bf16x3")
     tf32_peak = pk.get("bf16_tflops_sustained", 1700.0) * (1.0 if f16_kind else 1.1 / 2.25)
-    roof_g = {"bound": "alu", "kernel": "gather", "achieved": g_ach, "peak": fp32_peak, "unit": "TFLOP/s",
-              "frac": g_ach / fp32_peak, "traffic": None, "ms_per_launch": g_ms,
-              "peak_note": "FP32 FMA pipe: 152 SMs x 128 lanes x 2 FLOP x max SM clock (%s MHz)"
-                           % pk.get("sm_max_mhz", 2070.0),
-              "algorithmic_flop_per_pair": flop_pair, "algorithmic_note": GATHER_NOTE}
-    roof_c = {"bound": "tensor", "kernel": "contraction", "achieved": contraction_tflops, "peak": tf32_peak,
-              "unit": "TFLOP/s", "frac": (contraction_tflops or 0.0) / tf32_peak, "traffic": None,
+    roof_g = gather_roofline(pairs, nmax, sector_share, waves, bd["ms_gather"], fp32_peak)
+    roof_g["peak_note"] = ("FP32 FMA pipe: 152 SMs x 128 lanes x 2 FLOP x max SM clock (%s MHz)"
+                           % pk.get("sm_max_mhz", 2070.0))
+    issued = issued_flop(args.precision, bd["centres"], nmax, nb)
+    issued_tflops = issued / (bd["ms_contract"] / 1e3) / 1e12 if bd["ms_contract"] > 0 else None
+    roof_c = {"bound": "tensor", "kernel": "contraction", "achieved": issued_tflops, "peak": tf32_peak,
+              "unit": "TFLOP/s", "frac": (issued_tflops or 0.0) / tf32_peak, "traffic": None,
               "ms_per_launch": c_ms,
-              "passes": passes,
+              "passes": passes, "algorithmic_tflops": contraction_tflops,
+              "achieved_note": "operations issued: all passes, in the f16x3 form the padding of the tiles too",
               "peak_note": ("kind::f16 dense: measured sustained bf16 (%s TFLOP/s, %s)"
                             % (pk.get("bf16_tflops_sustained"), pk.get("source"))) if f16_kind else
                            ("tf32 dense: measured sustained bf16 (%s TFLOP/s, %s) x the nominal ratio 1.1/2.25 "
@@ -574,9 +627,9 @@ def run_ours(args):
     # DRAM bytes (read + write) of one full-size launch of the default configuration, from the
     # committed ncu summaries (null when the kernel source changed since the capture)
     if args.n_gal is None and args.centres is None:
-        roof_g["traffic"] = measured_traffic("gather_sector_kernel")
+        roof_g["traffic"] = measured_traffic("gather_sector_kernel") if sector_share > 0.5 else None
         roof_c["traffic"] = measured_traffic("contract_h16_kernel" if args.precision == "f16x3"
-                                             else "contract_tc_kernel" if tc_form else "contract_kernel")
+                                             else "contract_tc_kernel" if tc_form else "contract_rows")
         roof_g["traffic_unit"] = roof_c["traffic_unit"] = "bytes per launch (DRAM read + write, ncu)"
     roof_main, roof_other = (roof_c, roof_g) if c_ms >= g_ms else (roof_g, roof_c)
 
@@ -807,19 +860,18 @@ def run_batched(args, kind):
 
     # rooflines of the two dominant kernels from the steady-state call's phase times
     waves = max(1, bd["waves"])
-    flop_pair = gather_flop_per_pair(nmax)
-    g_ms = bd["ms_gather"] / waves
-    g_ach = flop_pair * pairs / (bd["ms_gather"] / 1e3) / 1e12
     fp32_peak = N_SM * FP32_LANES_PER_SM * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
     c_flop = reduced_contraction_flop(bd["centres"], nmax, nb)
     c_tflops = c_flop / (bd["ms_contract"] / 1e3) / 1e12 if bd["ms_contract"] > 0 else None
     peak_c = pk.get("bf16_tflops_sustained", 1700.0)
-    roof_g = {"bound": "alu", "kernel": "gather", "achieved": g_ach, "peak": fp32_peak, "unit": "TFLOP/s",
-              "frac": g_ach / fp32_peak, "traffic": None, "ms_per_launch": g_ms,
-              "peak_note": "FP32 FMA pipe: 152 SMs x 128 lanes x 2 FLOP x max SM clock",
-              "algorithmic_flop_per_pair": flop_pair, "algorithmic_note": GATHER_NOTE}
-    roof_c = {"bound": "tensor", "kernel": "contraction", "achieved": c_tflops, "peak": peak_c, "unit": "TFLOP/s",
-              "frac": (c_tflops or 0.0) / peak_c, "passes": 3,
+    sector_share = ext4pcf.ext4pcf_sector_centres(ctx) / max(1.0, bd["centres"])
+    roof_g = gather_roofline(pairs, nmax, sector_share, waves, bd["ms_gather"], fp32_peak)
+    roof_g["peak_note"] = "FP32 FMA pipe: 152 SMs x 128 lanes x 2 FLOP x max SM clock"
+    issued = issued_flop(args.precision, bd["centres"], nmax, nb)
+    issued_tflops = issued / (bd["ms_contract"] / 1e3) / 1e12 if bd["ms_contract"] > 0 else None
+    roof_c = {"bound": "tensor", "kernel": "contraction", "achieved": issued_tflops, "peak": peak_c, "unit": "TFLOP/s",
+              "frac": (issued_tflops or 0.0) / peak_c, "passes": 3, "algorithmic_tflops": c_tflops,
+              "achieved_note": "operations issued: all passes, in the f16x3 form the padding of the tiles too",
               "traffic": None, "ms_per_launch": bd["ms_contract"] / waves,
               "peak_note": "kind::f16 dense: measured sustained bf16 (%s TFLOP/s, %s)"
                            % (pk.get("bf16_tflops_sustained"), pk.get("source")),

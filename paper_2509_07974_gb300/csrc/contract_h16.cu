@@ -3,7 +3,7 @@
 // The GEMM runs over the independent sums of basis.cuh: for fixed sg the row products
 // G_a(b2) G_{sg-a}(b3), b2 <= b3, are multiplied with the columns x G_{-sg-8}(b1), x^* G_{-sg-4}(b1),
 // x G_{sg+4}^*(b1) and x^* G_sg^*(b1) (families F0..F3; W rows with the column w W_{-sg}), K running
-// over the centres.  Every row product serves four families, so 1643 tiles of 128 rows (n_max = 20,
+// over the centres.  Every row product serves four families, so 1655 tiles of 128 rows (n_max = 20,
 // 10 bins) hold what took 5572 tiles with a row type per component.  Forming the rows on the CUDA
 // cores is the larger part of the work.  One wave of 8192 centres at these sizes: 6.5 -> 2.24 ms
 // (3300 clocks per 64-centre stage of a tile; by count of its accesses shared memory is busy for about 2750
