@@ -60,9 +60,6 @@ template <> struct Pair<double> {
     double rinv = 1.0 / sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
     ur = dx * rinv; ui = dy * rinv;
   }
-  __device__ static void load_x(const SortedCat& cat, int q, double& xr, double& xi, double& w) {
-    xr = cat.xr[q]; xi = cat.xi[q]; w = cat.w[q];
-  }
 };
 
 template <> struct Pair<float> {
