@@ -50,3 +50,33 @@ def test_slots_share_the_sums_of_the_forms_that_take_them_in_turn(torch_cuda):  
         took[n_out] = _taken(torch, lambda est: ext4pcf.ext4pcf_measure_batch(
             est.ctx, *cat, n, edges, nb, nmax, offs, 8, slots, n_out, None, ups))
     assert took[8] <= took[1] + (16 << 20), took
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5), ("f16x3", 1e-5), ("3xtf32", 1e-5)])
+def test_xi_of_alternating_slots(torch_cuda, prec, tol):  # noqa: F811
+    """The xi accumulators of four catalogues in two slots, in turn, against the pair sums written out: sums
+    of FP32 records, (2 m + 16) 2^-23 of the absolute sum with m <= 4 (3e-6), in FP64 2^-52."""
+    from paper_2509_07974_gb300 import ext4pcf
+    torch, nb, n = torch_cuda, 3, 120
+    rng, edges = np.random.default_rng(9), np.geomspace(0.4, 4.0, nb + 1)
+    pos, sh, w = rng.uniform(0, 8, (4 * n, 2)), rng.normal(0, 0.3, (4 * n, 2)), rng.uniform(0.5, 1.5, 4 * n)
+    offs, slots = np.arange(5, dtype=np.int64) * n, np.array([1, 0, 1, 0], dtype=np.int32)
+    ups = torch.zeros(ext4pcf.Estimator.ups_shape(nb, 2, 2), dtype=torch.float64, device="cuda:0")
+    xi = torch.zeros((2, nb, 3, 2), dtype=torch.float64, device="cuda:0")
+    est = ext4pcf.Estimator(0, prec)
+    t = [torch.tensor(a, device="cuda:0") for a in (pos, sh, w)]
+    ext4pcf.ext4pcf_measure_batch(est.ctx, *t, 4 * n, edges, nb, 2, offs, 4, slots, 2, None, ups, xi)
+    got = torch.view_as_complex(xi).cpu().numpy()
+    est.close()
+    want, size = np.zeros((2, nb, 3), complex), np.zeros((2, nb, 3))
+    for k in range(4):
+        s = slice(k * n, (k + 1) * n)
+        d = pos[s][None] - pos[s][:, None]
+        r2, u = (d ** 2).sum(-1), np.exp(1j * np.arctan2(d[..., 1], d[..., 0]))
+        x, ww = w[s] * (sh[s, 0] + 1j * sh[s, 1]), w[s]
+        for b in range(nb):
+            m = (r2 >= edges[b] ** 2) & (r2 < edges[b + 1] ** 2)
+            for q, v in enumerate((x.conj()[:, None] * x[None], x[:, None] * x[None] * u ** -4, ww[:, None] * ww[None])):
+                want[slots[k], b, q] += v[m].sum()
+                size[slots[k], b, q] += np.abs(v[m]).sum()
+    assert (np.abs(got - want) <= tol * size).all(), np.abs(got - want).max()
