@@ -3,7 +3,7 @@
 //
 // One block takes one sg and one slice of the wave's centres.  It stages the two merged factors XX_sg
 // and XA_{sg+4} and the four columns x G_{-sg-8}, x^* G_{-sg-4}, x G_{sg+4}^*, x^* G_sg^* of 32 centres
-// (each loaded once for the six arrays they serve), and a thread holds a 2 x 2 tile of bins of one
+// (corr_chunk; each loaded once for the six arrays they serve), and a thread holds a 2 x 2 tile of bins of one
 // array, or with few bins its part of the centres.  Products and sums over corr_run centres are in R,
 // the rest in FP64; every slice adds into a copy of its own (one writer, no atomics), and the copies
 // are added in order at the end of the call.
@@ -18,17 +18,17 @@ namespace ext4pcf {
 
 namespace {
 
-constexpr int kCorrChunk = 32;  // centres staged at once
-
 // Few bins have few tiles: up to kCorrParts threads share one, each with every parts-th centre.
 constexpr int kCorrParts = 8;
 // Centres that a thread sums in FP32 before it adds them in FP64.  Few bins are the cheaper ones and keep
-// more of their sums in FP64: no more than the 1, 3, 7, 11, 19 ... centres that 192 threads sharing the
-// tiles of 2, 4, 6, 8, 10 ... bins have of 128 each.  (16 for every number of bins lost what lies 2^-24 below the
-// largest of 16 terms.)  Whole split-FP16 calls on 3000 galaxies with 16 everywhere, with these runs and one
-// thread to a tile, and as it is: 0.72, 1.07, 0.78 ms (2 bins, n_max = 20); 0.57, 0.67, 0.61 ms (4, 10);
-// 1.03, 1.13, 1.09 ms (5, 20).
-__host__ __device__ constexpr int corr_run(int nb) { return nb <= 2 ? 1 : nb <= 4 ? 2 : nb <= 6 ? 6 : nb <= 8 ? 8 : 16; }
+// more of their sums in FP64: the 1, 3, 7, 11 centres that 192 threads sharing the tiles of 2, 4, 6, 8
+// bins have of 128 each (at 10 bins and more it would be 19 and up).  16 for every number of bins lost what lies 2^-24
+// below the largest of 16 terms.  Whole split-FP16 calls on 3000 galaxies with 16 everywhere, with runs of 1, 2, 4,
+// 8 and one thread to a tile, and as it is: 0.72, 1.07, 0.77 ms (2 bins, n_max = 20); 0.57, 0.67, 0.59 ms
+// (4, 10); 1.03, 1.13, 1.06 ms (5, 20).
+__host__ __device__ constexpr int corr_run(int nb) { return nb <= 2 ? 1 : nb <= 4 ? 3 : nb <= 6 ? 7 : nb <= 8 ? 11 : 16; }
+// Centres staged at once: two full runs of every thread that shares a tile (8, 3, 2 of them for 4, 6, 8 bins)
+__host__ __device__ constexpr int corr_chunk(int nb) { return nb <= 2 ? 32 : nb <= 4 ? 48 : nb <= 6 ? 42 : nb <= 8 ? 44 : 32; }
 
 template <typename Cx> struct __align__(16) Pair2 { Cx a, b; };
 
@@ -107,8 +107,8 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
   const int sg = wk ? job - C.nsig : -2 * N - 6 + job;  // (W blocks: the index c)
   const int width = (wk ? 2 : 6) * nbp;                 // staged values per centre
   const int tiles = (wk ? 1 : 6) * nt * nt;
-  const int run = SHARED && sizeof(R) == 4 ? corr_run(nb) : 16;
-  Cx* st = reinterpret_cast<Cx*>(smem_raw);  // [kCorrChunk][width]
+  const int run = SHARED && sizeof(R) == 4 ? corr_run(nb) : 16, chunk = SHARED ? corr_chunk(nb) : 32;
+  Cx* st = reinterpret_cast<Cx*>(smem_raw);  // [chunk][width]
   // the value this thread stages of every (blockDim / width)-th centre: its place in a record (-1: a
   // zero), its conjugation and its centre factor (0: none, 1: x, 2: x^*, 3: w)
   const int cper = blockDim.x / width, scol = tid % width, scc = tid / width;
@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(384) corrections_kernel(const Layout L, const 
       double a64[4][2];
 #pragma unroll
       for (int i = 0; i < 4; ++i) a64[i][0] = a64[i][1] = 0.0;
-      for (int c0 = t0; c0 < t1; c0 += kCorrChunk) {
-        const int nc = min(kCorrChunk, t1 - c0);
+      for (int c0 = t0; c0 < t1; c0 += chunk) {
+        const int nc = min(chunk, t1 - c0);
         __syncthreads();
         if (scc < cper) {
 #pragma unroll 4
@@ -270,7 +270,7 @@ cudaError_t corrections_wave(const Layout& L, const cplx_t<R>* rec, const cplx_t
   // up to eight bins 192 threads: 8, 8, 3 and 2 to a tile of the six X arrays
   const bool shared = nt <= 4;
   const int threads = std::min(384, std::max(shared ? 192 : 160, (6 * nt * nt + 31) / 32 * 32));
-  const size_t smem = std::max((size_t)kCorrChunk * 12 * nt * sizeof(cplx_t<R>),
+  const size_t smem = std::max((size_t)corr_chunk(L.nb) * 12 * nt * sizeof(cplx_t<R>),
                                (size_t)threads * (shared ? 4 : 1) * sizeof(double2));
   auto kernel = shared ? corrections_kernel<R, true> : corrections_kernel<R, false>;
   cudaError_t e = allow_smem(kernel);
